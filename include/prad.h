@@ -95,7 +95,11 @@ typedef struct prad_config {
   int32_t sort_interval;    /* YEE2D with a pid array: reorder particles by
                                32 x 32-cell tile (and cell) every this many
                                steps and gather from shared-memory field
-                               tiles (0 = never sort; plain gather)       */
+                               tiles (0 = particles stay in the caller's
+                               order: long FP32 calls gather through tiles
+                               from a reordered copy, 44 B x max_particles
+                               of context scratch, short ones from the
+                               planes)                                    */
   int32_t batch_chunk;      /* push_emit_batch: particles per work item
                                (0 = 2048); multiple of 32                 */
   int32_t use_graph;        /* push_emit_batch: capture the launches of a

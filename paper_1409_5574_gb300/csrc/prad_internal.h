@@ -151,6 +151,12 @@ struct StepParams {
   const int4* work;           // (tile, first, end, 0) per work item
   const unsigned int* work_count;
   int32_t ntx;                // tiles along x
+  // binned Yee gather (particles stay in the caller's order): the state in
+  // tile and cell order, two vectors per particle, (x, y, z, u_x) and
+  // (u_y, u_z, w, id as bits); the plain kernel that stands behind it runs
+  // only where *gate is not 0
+  float4* aos;
+  const unsigned int* gate;
   // Philox4x32-10 round keys of (key0, key1) (philox_round_keys), read
   // from the kernel's parameter space by the kernels that take StepParams
   // by value
@@ -163,7 +169,8 @@ constexpr int kTile = 32;
 constexpr int kHalo = 6;
 constexpr int kStageW = kTile + 2 * kHalo;
 constexpr int kTileSmemBytes = 6 * kStageW * kStageW * 4;
-constexpr int kChunk = 4096;  // particles per work item of the tiled kernel
+constexpr int kChunk = 4096;     // particles per work item of the tiled kernel at most
+constexpr int kChunkMin = 512;   // and at least (sizes the work list)
 
 struct SortBuffers {
   void* tmp[7];               // scratch copies of x y z ux uy uz w
@@ -175,6 +182,22 @@ struct SortBuffers {
   unsigned int* work_count;
   int64_t capacity;           // particles
   int32_t ntiles, max_work;
+};
+
+// Scratch of the binned Yee gather: (particle, cell) keys in tile order, each
+// particle's slot in the order by tile and cell, the state in that order, tile
+// counters, the work list and the gate.
+struct BinBuffers {
+  uint2* keys;
+  uint32_t* slot;
+  float4* aos;                // two per particle
+  unsigned int* counts;       // per tile
+  unsigned int* starts;       // per tile + 1
+  unsigned int* cursor;       // per tile
+  int4* work;
+  unsigned int* work_count;   // [0] work items, [1] gate of the plain kernel
+  int64_t capacity;           // particles
+  int32_t ntiles;
 };
 
 // Batched ensembles (k_push_emit_batch): per-ensemble step parameters in a
@@ -226,13 +249,21 @@ cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
                                 R* x_out, R* g_out, int64_t n, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
                           uint32_t* out, int64_t n, cudaStream_t s);
+// (p.aos: the binned form)
 template <typename R>
 cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int block,
                                    cudaStream_t s);
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,
                              int nx, int ny, double x0, double y0, double inv_dx,
-                             double inv_dy, cudaStream_t s);
+                             double inv_dy, int chunk, cudaStream_t s);
+// The state of the p.n particles of p into b.aos in the order of their tiles
+// and cells, and the work list (chunks of at most `chunk` particles of one
+// tile); launch_tile_unbin writes it back to where it came from.
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
+                            double inv_dx, double inv_dy, int chunk, int num_sms, cudaStream_t s);
+cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, int num_sms,
+                              cudaStream_t s);
 size_t mlp_train_smem_bytes();
 cudaError_t launch_mlp_train_block(const MlpDev& dev, uint32_t key0, uint32_t key1,
                                    uint64_t first, int64_t n_valid, int64_t n_total,
@@ -292,7 +323,7 @@ cudaError_t launch_ledger_reduce(const double* a, const double* b, int64_t n,
 // Run-time specialised kernels (spec.cu): the standard FP32 plane-wave and
 // Yee-grid step kernels compiled by NVRTC with the context's constants as
 // literals.  A variant names the kernel (k_push_emit, or k_push_emit_tiled
-// when tiled), field model, sampler, prefetch mode and plane-wave signs.
+// when tiled, 2 its binned form), field model, sampler, prefetch mode and plane-wave signs.
 // spec_get returns its kernel for these parameters' constants, compiling it
 // on first use (an error, with a message in msg, when NVRTC or the driver
 // cannot provide it).

@@ -856,6 +856,21 @@ __device__ __forceinline__ void load_state(const StepParams<R>& P, int64_t i, bo
   }
 }
 
+// The same from the binned state (two vectors per particle).
+__device__ __forceinline__ void load_aos(const StepParams<float>& P, int64_t i, bool act,
+                                         PState<float>& s) {
+  float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+  if (act) {
+    a = P.aos[2 * i];
+    b = P.aos[2 * i + 1];
+  }
+  s.act = act;
+  s.x = a.x; s.y = a.y; s.z = a.z;
+  s.ux = a.w; s.uy = b.x; s.uz = b.y; s.w = b.z;
+  s.pid = __float_as_uint(b.w);
+  s.ll_old = s.emit_old = 0.0;
+}
+
 // One-step launches of the FP32 table sampler without control read the
 // sampling table from a copy in shared memory (advance_particle's STAB):
 // there the streamed state passes through L1 and would evict it.  (Fused
@@ -878,11 +893,13 @@ constexpr bool kSharedTab =
 // CTRL: super-photon control or diagnostics are enabled (the plain method
 // compiles without their per-step work).
 // rk: the Philox round keys, in the kernel's parameter space.
+// AOS: the state is P.aos, two vectors per particle (binned Yee launches).
 // STD: the standard configuration (LL kick applied, field form of H_eff,
 // three dimensions, two for the Yee grid) fixed at compile time, so the step
 // tests no mode.
 template <typename R, int FIELD, int SAMP, int ONE = 0, int CTRL = 0,
-          bool STD = false, bool STAB = false, int PWS = 0, class G, class ST>
+          bool STD = false, bool STAB = false, int PWS = 0, bool AOS = false, class G,
+          class ST>
 __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const uint32_t (&rk)[20],
                                                  const G& gat,
                                                  int64_t i, const PState<R>& st,
@@ -1134,9 +1151,14 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
     ux = nux; uy = nuy; uz = nuz;
   }
   if (live) {
-    P.x[i] = x; P.y[i] = y;
-    if (P.z) P.z[i] = z;
-    P.ux[i] = ux; P.uy[i] = uy; P.uz[i] = uz;
+    if constexpr (AOS) {
+      P.aos[2 * i] = make_float4(x, y, z, ux);
+      P.aos[2 * i + 1] = make_float4(uy, uz, w, __uint_as_float(pid));
+    } else {
+      P.x[i] = x; P.y[i] = y;
+      if (P.z) P.z[i] = z;
+      P.ux[i] = ux; P.uy[i] = uy; P.uz[i] = uz;
+    }
     if constexpr (ONE == 2) {
       if (rr_mode >= PRAD_RR_LEDGER) P.led_ll[i] = st.ll_old + ll.value_one();
       // (with control a step may add several trials: the full value)
@@ -1303,6 +1325,9 @@ __global__ void __launch_bounds__(256, (PF ? PRAD_PF_MINB : MinBlocks<R, FIELD, 
 #else
   const StepParams<R>& P = P_arg;
 #endif
+  if constexpr (FIELD == PRAD_FIELD_YEE2D) {  // behind a binned launch
+    if (P.gate && *P.gate == 0u) return;
+  }
   constexpr bool kSTab = kSharedTab<R, SAMP, PF, CTRL>;
   using Stage = typename std::conditional<
       CTRL == 2, PhotonStageSpread,
@@ -1503,7 +1528,8 @@ int batch_max_blocks_per_sm(int block, int sampler, bool ctrl, bool std_cfg) {
 // (+ halo, periodic) in shared memory with coalesced row loads, then runs the
 // same per-particle path with the shared-memory gather.
 // ---------------------------------------------------------------------------
-template <typename R, int CTRL, bool STD = false>
+// AOS: the binned form, for particles kept in another order (P.aos).
+template <typename R, int CTRL, bool STD = false, bool AOS = false>
 __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> P_arg) {
 #ifdef PRAD_SPEC
   const StepParams<R> P = spec_params(P_arg);
@@ -1551,8 +1577,11 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   for (int64_t base = wk.y; base < wk.z; base += blockDim.x) {
     const int64_t i = base + threadIdx.x;
     PState<R> st;
-    load_state(P, i, i < wk.z, st);
-    advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD>(
+    if constexpr (AOS)
+      load_aos(P, i, i < wk.z, st);
+    else
+      load_state(P, i, i < wk.z, st);
+    advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, AOS>(
         P, P.rkey, gat, i, st, stage, fill, pout, cnt);
   }
   if (fill > 0) flush_stage(stage, fill, pout);
@@ -1573,15 +1602,22 @@ bool std_config(const StepParams<R>& p, int dims) {
          p.abs_q == R(1);
 }
 
-template <typename R, int CTRL, bool STD>
-cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
+template <typename R, int CTRL, bool STD, bool AOS>
+cudaError_t launch_tiled_a(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
   // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
-  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
+  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD, AOS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kTileSmemBytes);
   if (e != cudaSuccess) return e;
-  k_push_emit_tiled<R, CTRL, STD><<<max_work, block, kTileSmemBytes, s>>>(p);
+  k_push_emit_tiled<R, CTRL, STD, AOS><<<max_work, block, kTileSmemBytes, s>>>(p);
   return cudaGetLastError();
+}
+
+template <typename R, int CTRL, bool STD>
+cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
+  if constexpr (sizeof(R) == 4)
+    if (p.aos) return launch_tiled_a<R, CTRL, STD, true>(p, max_work, block, s);
+  return launch_tiled_a<R, CTRL, STD, false>(p, max_work, block, s);
 }
 
 template <typename R>
@@ -1740,7 +1776,7 @@ bool push_emit_spec_variant(const StepParams<float>& p, int field_kind, int samp
   if (ctrl) return false;
   v->field = field_kind;
   v->samp = sampler;
-  v->tiled = tiled ? 1 : 0;
+  v->tiled = tiled ? (p.aos ? 2 : 1) : 0;
   v->pf = 0;
   v->pws = 0;
   if (tiled) return field_kind == PRAD_FIELD_YEE2D && sampler == PRAD_SAMPLER_TABLE &&

@@ -69,6 +69,10 @@ __device__ __forceinline__ unsigned int warp_claim(unsigned int* counter, int t,
   return slot;
 }
 
+// Binned gather: below this many particles per occupied tile the plain kernel
+// gathers from global memory (a tile's staging would not pay).
+constexpr unsigned int kBinSparse = 64;
+
 // Grid-stride over warps of 32 consecutive particles (every lane of a warp
 // takes the same number of iterations).
 template <typename R>
@@ -88,48 +92,82 @@ __global__ void k_tile_count(const R* __restrict__ x, const R* __restrict__ y, i
 
 // One block: exclusive scan of the tile counts (starts, scatter cursors) and
 // of the per-tile chunk counts (work list offsets); writes the work list.
+// Warp w owns a contiguous run of tiles and reads it 32 at a time, so counts,
+// starts and cursors are touched in whole lines (one tile per thread and
+// iteration; with a run of tiles per thread 16384 tiles took 27 us, now 7).
 constexpr int kScanThreads = 1024;
 
+__device__ __forceinline__ unsigned int warp_inclusive(unsigned int v, int lane) {
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const unsigned int u = __shfl_up_sync(0xffffffffu, v, off);
+    if (lane >= off) v += u;
+  }
+  return v;
+}
+
+// sparse > 0 (binned gather): with fewer than `sparse` particles per occupied
+// tile there is no tile work, and the gate lets the plain kernel run instead.
 __global__ void __launch_bounds__(kScanThreads)
     k_tile_scan(const unsigned int* __restrict__ counts, int ntiles,
                 unsigned int* __restrict__ starts, unsigned int* __restrict__ cursor,
-                int4* __restrict__ work, unsigned int* __restrict__ work_count) {
-  __shared__ unsigned int s_part[kScanThreads], s_chunk[kScanThreads];
-  const int per = (ntiles + kScanThreads - 1) / kScanThreads;
-  const int lo = threadIdx.x * per;
-  const int hi = min(lo + per, ntiles);
-  unsigned int sum = 0, csum = 0;
-  for (int t = lo; t < hi; ++t) {
-    sum += counts[t];
-    csum += (counts[t] + kChunk - 1) / kChunk;
+                int4* __restrict__ work, unsigned int* __restrict__ work_count,
+                unsigned int chunk, unsigned int sparse) {
+  constexpr int kWarps = kScanThreads / 32;
+  __shared__ unsigned int s_sum[kWarps], s_chunks[kWarps], s_used[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = ((ntiles + kWarps - 1) / kWarps + 31) / 32 * 32;
+  const int lo = warp * per, hi = min(lo + per, ntiles);
+  unsigned int sum = 0, chunks = 0, used = 0;
+#pragma unroll 4
+  for (int t0 = lo; t0 < hi; t0 += 32) {
+    const unsigned int c = t0 + lane < hi ? counts[t0 + lane] : 0u;
+    sum += c;
+    chunks += (c + chunk - 1) / chunk;
+    used += c != 0u;
   }
-  s_part[threadIdx.x] = sum;
-  s_chunk[threadIdx.x] = csum;
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  chunks = __reduce_add_sync(0xffffffffu, chunks);
+  used = __reduce_add_sync(0xffffffffu, used);
+  if (lane == 0) {
+    s_sum[warp] = sum;
+    s_chunks[warp] = chunks;
+    s_used[warp] = used;
+  }
   __syncthreads();
-  // Hillis-Steele inclusive scan over the thread partials
-  for (int off = 1; off < kScanThreads; off <<= 1) {
-    const unsigned int a = threadIdx.x >= off ? s_part[threadIdx.x - off] : 0u;
-    const unsigned int b = threadIdx.x >= off ? s_chunk[threadIdx.x - off] : 0u;
-    __syncthreads();
-    s_part[threadIdx.x] += a;
-    s_chunk[threadIdx.x] += b;
-    __syncthreads();
-  }
-  unsigned int run = s_part[threadIdx.x] - sum;
-  unsigned int wrun = s_chunk[threadIdx.x] - csum;
-  for (int t = lo; t < hi; ++t) {
-    const unsigned int c = counts[t];
-    starts[t] = run;
-    cursor[t] = run;
-    for (unsigned int f = 0; f < c; f += kChunk) {
-      const unsigned int e = f + kChunk < c ? f + kChunk : c;
-      work[wrun++] = make_int4(t, static_cast<int>(run + f), static_cast<int>(run + e), 0);
+  if (warp == 0) {
+    const unsigned int a = s_sum[lane], b = s_chunks[lane];
+    const unsigned int ia = warp_inclusive(a, lane), ib = warp_inclusive(b, lane);
+    const unsigned int tiles = __reduce_add_sync(0xffffffffu, s_used[lane]);
+    s_sum[lane] = ia - a;
+    s_chunks[lane] = ib - b;
+    if (lane == 31) {
+      starts[ntiles] = ia;
+      const bool none = sparse != 0u && ia < static_cast<uint64_t>(sparse) * tiles;
+      work_count[0] = none ? 0u : ib;
+      if (sparse != 0u) work_count[1] = none ? 1u : 0u;
     }
-    run += c;
   }
-  if (threadIdx.x == kScanThreads - 1) {
-    starts[ntiles] = run;
-    *work_count = wrun;
+  __syncthreads();
+  unsigned int run = s_sum[warp], wrun = s_chunks[warp];
+#pragma unroll 4
+  for (int t0 = lo; t0 < hi; t0 += 32) {
+    const int t = t0 + lane;
+    const unsigned int c = t < hi ? counts[t] : 0u;
+    const unsigned int k = (c + chunk - 1) / chunk;
+    const unsigned int ic = warp_inclusive(c, lane), ik = warp_inclusive(k, lane);
+    const unsigned int first = run + ic - c;
+    if (t < hi) {
+      starts[t] = first;
+      cursor[t] = first;
+    }
+    unsigned int w = wrun + ik - k;
+    for (unsigned int f = 0; f < c; f += chunk) {
+      const unsigned int e = f + chunk < c ? f + chunk : c;
+      work[w++] = make_int4(t, static_cast<int>(first + f), static_cast<int>(first + e), 0);
+    }
+    run += __shfl_sync(0xffffffffu, ic, 31);
+    wrun += __shfl_sync(0xffffffffu, ik, 31);
   }
 }
 
@@ -217,12 +255,253 @@ __global__ void __launch_bounds__(kCellThreads)
   }
 }
 
+// ---------------------------------------------------------------------------
+// Binning: a copy of the state in the same order (tile, then cell), for
+// particles that stay where the caller keeps them.  The caller's arrays are
+// only ever streamed; the scattered side is the copy, whose particles are
+// one 32-byte sector each.  (Gathering the seven arrays through an index in
+// the push itself cost 0.25 ns per particle and launch on 8M particles in
+// random order; now 2^21 particles in random order take 13 us to count, 6 to
+// scan, 27 + 28 to place by tile and cell, 39 to copy and 26 to write back,
+// beside 1014 us for 25 steps of the push: 7.98 ms with the plain gather,
+// 1.38 ms so.)  Block b owns the contiguous
+// particles [n b / B, n (b + 1) / B); the tile counters of its particles sit
+// in shared memory (SM) so that a tile costs a block one global atomic, not
+// one per warp that meets it; grids of more than kBinTiles tiles count in
+// global memory.
+// ---------------------------------------------------------------------------
+constexpr int kBinThreads = 512;
+constexpr int kBinTiles = 16384;  // 64 KB of shared counters
+
+struct BinGeom {
+  int nx, ny, ntx, ntiles;
+  float x0, y0, inv_dx, inv_dy;
+};
+
+__device__ __forceinline__ uint2 bin_of(const BinGeom& g, float x, float y) {
+  const int2 c = cell_xy(x, y, g.nx, g.ny, g.x0, g.y0, g.inv_dx, g.inv_dy);
+  return make_uint2(static_cast<unsigned>((c.y / kTile) * g.ntx + (c.x / kTile)),
+                    static_cast<unsigned>((c.y % kTile) * kTile + (c.x % kTile)));
+}
+
+// An increment of tile t's counter by every valid lane and the slot it got.
+// Shared counters: one add for a warp inside one tile, else one per lane
+// (grouping the lanes of a warp by tile costs more than the adds when the
+// caller's order is random); global ones: one add per tile of the warp.
+template <bool SM>
+__device__ __forceinline__ unsigned int bin_claim(unsigned int* cnt, unsigned int t, bool valid) {
+  if constexpr (!SM) return warp_claim(cnt, static_cast<int>(t), valid);
+  const int lane = threadIdx.x & 31;
+  unsigned int d = 0u;
+  const unsigned int t0 = __shfl_sync(0xffffffffu, t, 0);  // (by every lane, valid or not)
+  const bool same = valid && t == t0;
+  if (__all_sync(0xffffffffu, same)) {
+    if (lane == 0) d = atomicAdd(cnt + t, 32u);
+    return __shfl_sync(0xffffffffu, d, 0) + lane;
+  }
+  if (valid) d = atomicAdd(cnt + t, 1u);
+  return d;
+}
+
+// Counts of this block's particles by tile, added into cnt.
+template <bool SM>
+__device__ __forceinline__ void bin_count_range(const BinGeom& g, const float* __restrict__ x,
+                                                const float* __restrict__ y, int64_t lo,
+                                                int64_t hi, unsigned int* cnt) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 4
+  for (int64_t w0 = lo + (threadIdx.x & ~31); w0 < hi; w0 += kBinThreads) {
+    const int64_t i = w0 + lane;
+    const bool valid = i < hi;
+    const unsigned t = valid ? bin_of(g, x[i], y[i]).x : 0u;
+    (void)bin_claim<SM>(cnt, t, valid);
+  }
+}
+
+template <bool SM>
+__global__ void __launch_bounds__(kBinThreads)
+    k_bin_count(const BinGeom g, const float* __restrict__ x, const float* __restrict__ y,
+                int64_t n, unsigned int* __restrict__ counts) {
+  extern __shared__ unsigned int s_tile[];
+  const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
+  if constexpr (SM) {
+    for (int t = threadIdx.x; t < g.ntiles; t += kBinThreads) s_tile[t] = 0u;
+    __syncthreads();
+    bin_count_range<true>(g, x, y, lo, hi, s_tile);
+    __syncthreads();
+    for (int t = threadIdx.x; t < g.ntiles; t += kBinThreads)
+      if (s_tile[t]) atomicAdd(counts + t, s_tile[t]);
+  } else {
+    bin_count_range<false>(g, x, y, lo, hi, counts);
+  }
+}
+
+// Keys (particle, cell) into tile order.  SM: the block counts its particles
+// again, reserves its run of every tile it meets with one atomic, and places
+// them with shared cursors.
+template <bool SM>
+__global__ void __launch_bounds__(kBinThreads)
+    k_bin_scatter(const BinGeom g, const float* __restrict__ x, const float* __restrict__ y,
+                  int64_t n, unsigned int* __restrict__ cursor, uint2* __restrict__ keys) {
+  extern __shared__ unsigned int s_tile[];
+  const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
+  if constexpr (SM) {
+    for (int t = threadIdx.x; t < g.ntiles; t += kBinThreads) s_tile[t] = 0u;
+    __syncthreads();
+    bin_count_range<true>(g, x, y, lo, hi, s_tile);
+    __syncthreads();
+    for (int t = threadIdx.x; t < g.ntiles; t += kBinThreads)
+      if (s_tile[t]) s_tile[t] = atomicAdd(cursor + t, s_tile[t]);
+    __syncthreads();
+  }
+  unsigned int* cur = SM ? s_tile : cursor;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 4
+  for (int64_t w0 = lo + (threadIdx.x & ~31); w0 < hi; w0 += kBinThreads) {
+    const int64_t i = w0 + lane;
+    const bool valid = i < hi;
+    const uint2 b = valid ? bin_of(g, x[i], y[i]) : make_uint2(0u, 0u);
+    const unsigned int d = bin_claim<SM>(cur, b.x, valid);
+    if (valid) keys[d] = make_uint2(static_cast<unsigned>(i), b.y);
+  }
+}
+
+// One block per tile: the slots of the tile's particles in cell order.
+__global__ void __launch_bounds__(kBinThreads)
+    k_bin_cells(const uint2* __restrict__ keys, uint32_t* __restrict__ slot,
+                const unsigned int* __restrict__ starts) {
+  constexpr int kCells = kTile * kTile;
+  static_assert(kCells == 2 * kBinThreads, "two cells per thread");
+  __shared__ unsigned int s_cnt[kCells];
+  __shared__ unsigned int s_warp[kBinThreads / 32];
+  const unsigned int a = starts[blockIdx.x], b = starts[blockIdx.x + 1];
+  if (a == b) return;  // the whole block leaves
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  s_cnt[tid] = 0u;
+  s_cnt[tid + kBinThreads] = 0u;
+  __syncthreads();
+  for (unsigned int k = a + tid; k < b; k += kBinThreads) atomicAdd(s_cnt + keys[k].y, 1u);
+  __syncthreads();
+  // exclusive scan, thread tid holding cells 2 tid and 2 tid + 1
+  const unsigned int c0 = s_cnt[2 * tid], c1 = s_cnt[2 * tid + 1];
+  const unsigned int v = warp_inclusive(c0 + c1, lane);
+  if (lane == 31) s_warp[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    const unsigned int w = warp_inclusive(lane < kBinThreads / 32 ? s_warp[lane] : 0u, lane);
+    if (lane < kBinThreads / 32) s_warp[lane] = w;
+  }
+  __syncthreads();
+  const unsigned int e0 = (warp > 0 ? s_warp[warp - 1] : 0u) + v - c0 - c1;
+  s_cnt[2 * tid] = e0;
+  s_cnt[2 * tid + 1] = e0 + c0;
+  __syncthreads();
+  for (unsigned int k = a + tid; k < b; k += kBinThreads) {
+    const uint2 q = keys[k];
+    slot[q.x] = a + atomicAdd(s_cnt + q.y, 1u);
+  }
+}
+
+// The state to its slots, and back.
+__global__ void __launch_bounds__(256)
+    k_bin_pack(const StepParams<float> P, const uint32_t* __restrict__ slot,
+               const unsigned int* __restrict__ gate, float4* __restrict__ aos) {
+  if (*gate) return;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < P.n;
+       i += stride) {
+    const size_t d = slot[i];
+    const uint32_t id = P.pid ? P.pid[i] : P.pid0 + static_cast<uint32_t>(i);
+    aos[2 * d] = make_float4(P.x[i], P.y[i], P.z ? P.z[i] : 0.0f, P.ux[i]);
+    aos[2 * d + 1] = make_float4(P.uy[i], P.uz[i], P.w[i], __uint_as_float(id));
+  }
+}
+// (z and w do not change on the grid)
+__global__ void __launch_bounds__(256)
+    k_bin_unpack(const StepParams<float> P, const uint32_t* __restrict__ slot,
+                 const unsigned int* __restrict__ gate, const float4* __restrict__ aos) {
+  if (*gate) return;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < P.n;
+       i += stride) {
+    const size_t d = slot[i];
+    const float4 a = aos[2 * d], b = aos[2 * d + 1];
+    P.x[i] = a.x;
+    P.y[i] = a.y;
+    P.ux[i] = a.w;
+    P.uy[i] = b.x;
+    P.uz[i] = b.y;
+  }
+}
+
+int stream_grid(int64_t n, int num_sms) {
+  const int64_t want = (n + 255) / 256, cap = 8 * static_cast<int64_t>(num_sms);
+  return static_cast<int>(want < cap ? want : cap);
+}
+
 }  // namespace
+
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
+                            double inv_dx, double inv_dy, int chunk, int num_sms,
+                            cudaStream_t s) {
+  const int64_t n = p.n;
+  const float *x = p.x, *y = p.y;
+  BinGeom g;
+  g.nx = p.nx;
+  g.ny = p.ny;
+  g.ntx = (p.nx + kTile - 1) / kTile;
+  g.ntiles = b.ntiles;
+  g.x0 = static_cast<float>(x0);
+  g.y0 = static_cast<float>(y0);
+  g.inv_dx = static_cast<float>(inv_dx);
+  g.inv_dy = static_cast<float>(inv_dy);
+  cudaError_t e = cudaMemsetAsync(b.counts, 0, sizeof(unsigned int) * b.ntiles, s);
+  if (e != cudaSuccess) return e;
+  const bool sm = b.ntiles <= kBinTiles;
+  const size_t dyn = sm ? sizeof(unsigned int) * b.ntiles : 0;
+  if (dyn > 48 * 1024) {
+    if ((e = cudaFuncSetAttribute(k_bin_count<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kBinTiles * 4)) != cudaSuccess)
+      return e;
+    if ((e = cudaFuncSetAttribute(k_bin_scatter<true>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kBinTiles * 4)) != cudaSuccess)
+      return e;
+  }
+  // blocks: three per SM (64 KB of counters each at most), fewer for sets
+  // that would leave a block less than 2048 particles
+  const int64_t want = (n + 2047) / 2048;
+  const int grid = static_cast<int>(want < 3 * num_sms ? want : 3 * num_sms);
+  if (sm)
+    k_bin_count<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.counts);
+  else
+    k_bin_count<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.counts);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_tile_scan<<<1, kScanThreads, 0, s>>>(b.counts, b.ntiles, b.starts, b.cursor, b.work,
+                                          b.work_count, static_cast<unsigned int>(chunk),
+                                          kBinSparse);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (sm)
+    k_bin_scatter<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.cursor, b.keys);
+  else
+    k_bin_scatter<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.cursor, b.keys);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_bin_cells<<<b.ntiles, kBinThreads, 0, s>>>(b.keys, b.slot, b.starts);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  k_bin_pack<<<stream_grid(n, num_sms), 256, 0, s>>>(p, b.slot, b.work_count + 1, b.aos);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, int num_sms,
+                              cudaStream_t s) {
+  k_bin_unpack<<<stream_grid(p.n, num_sms), 256, 0, s>>>(p, b.slot, b.work_count + 1, b.aos);
+  return cudaGetLastError();
+}
 
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,
                              int nx, int ny, double x0, double y0, double inv_dx,
-                             double inv_dy, cudaStream_t s) {
+                             double inv_dy, int chunk, cudaStream_t s) {
   const int ntx = (nx + kTile - 1) / kTile;
   cudaError_t e = cudaMemsetAsync(b.counts, 0, sizeof(unsigned int) * b.ntiles, s);
   if (e != cudaSuccess) return e;
@@ -233,7 +512,7 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
                                          R(inv_dx), R(inv_dy), b.counts);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_tile_scan<<<1, kScanThreads, 0, s>>>(b.counts, b.ntiles, b.starts, b.cursor, b.work,
-                                          b.work_count);
+                                          b.work_count, static_cast<unsigned int>(chunk), 0u);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   Arrays7<R> srcp, dstp;
   for (int k = 0; k < 7; ++k) {
@@ -250,10 +529,10 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
 }
 
 template cudaError_t launch_tile_sort<float>(float* [7], uint32_t*, int64_t, const SortBuffers&,
-                                             int, int, double, double, double, double,
+                                             int, int, double, double, double, double, int,
                                              cudaStream_t);
 template cudaError_t launch_tile_sort<double>(double* [7], uint32_t*, int64_t,
                                               const SortBuffers&, int, int, double, double,
-                                              double, double, cudaStream_t);
+                                              double, double, int, cudaStream_t);
 
 }  // namespace prad
