@@ -371,8 +371,9 @@ int prad_get_photons(prad_ctx* ctx, prad_photons* out, int64_t cap,
                      int64_t* n_out, int64_t* n_dropped, int32_t drain,
                      int32_t out_on_device);
 
-/* Totals of the per-particle ledgers over all max_particles entries, by a
- * deterministic two-pass Kahan-compensated FP64 reduction on the device:
+/* Totals of the per-particle ledgers over all max_particles entries, the
+ * exact sums of the FP64 entries rounded once (NaN if an entry is not
+ * finite), on the device:
  * *emitted = sum of k w x hbar omega_c, *rr_loss = sum of the LL loss, both
  * in m c^2 (multiply by m_e c^2 for joules).  Either output may be NULL.
  * s (may be NULL) receives the counters.  Synchronises the stream. */
@@ -488,19 +489,18 @@ int prad_angular_histogram(prad_ctx* ctx, const double axis[3], const double ref
  * synchronises the device and may fail once the pool holds the memory) is
  * not acceptable.  It needs no context.
  *
- * The same deterministic two-pass Kahan totals as prad_energy_budget, of
+ * The same exact totals as prad_energy_budget, of
  * two caller-owned device FP64 arrays emit[n] and rr[n] (for example the
  * caller's own per-particle ledgers), written to out[0] (sum of emit) and
  * out[1] (sum of rr), a caller-owned device array of 2 doubles, on `stream`
- * (cudaStream_t; NULL = default stream); asynchronous.  The per-block
- * partials live in a file-scope device array of 4096 x 4 doubles (128 KB,
- * held by every GPU that loads the library until the process exits), so
- * n is limited to 4096 x 65536 = 268435456 entries; larger n returns
- * PRAD_ERR_ARG.  No cudaMalloc, cudaFree or allocating library routine is
+ * (cudaStream_t; NULL = default stream); asynchronous.  The scratch
+ * is a file-scope device array (2 KB, held by every GPU that loads the
+ * library until the process exits).  n is limited to 4096 x 65536 =
+ * 268435456 entries; larger n returns PRAD_ERR_ARG.  No cudaMalloc, cudaFree or allocating library routine is
  * called.  The first call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current; make that first call
  * before any stream capture.  All calls share the array and it keeps the
- * last call's contents (each call writes every partial it reads), so calls
+ * last call's contents (each call zeroes it before it reads it), so calls
  * that overlap on the GPU race: order them on one stream or synchronise.
  * n == 0 writes zeros (emit and rr may then be NULL).  The device address
  * looked up by the first call stays in use for the life of the process:

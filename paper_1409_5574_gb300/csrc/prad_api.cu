@@ -57,9 +57,8 @@ struct prad_ctx {
   unsigned long long* d_cnt = nullptr;
   double* d_led_emit = nullptr;
   double* d_led_ll = nullptr;
-  double* d_partials = nullptr;
+  void* d_red = nullptr;
   double* d_sums = nullptr;
-  int red_blocks = 0;
   // host-side totals folded in at each drain
   int64_t drained_records = 0;
   int64_t drained_dropped = 0;
@@ -1057,8 +1056,7 @@ int prad_init(prad_ctx** out, const prad_config* cfg) {
   CKI(cudaMalloc(&c->d_led_ll, np * sizeof(double)));
   CKI(cudaMemset(c->d_led_emit, 0, np * sizeof(double)));
   CKI(cudaMemset(c->d_led_ll, 0, np * sizeof(double)));
-  c->red_blocks = 2 * c->num_sms;
-  CKI(cudaMalloc(&c->d_partials, 4 * c->red_blocks * sizeof(double)));
+  CKI(cudaMalloc(&c->d_red, kLedgerScratchBytes));
   CKI(cudaMalloc(&c->d_sums, 2 * sizeof(double)));
   // learned sampler: network, optimiser state, G^-1 table
   CKI(cudaMalloc(&c->d_mlp, sizeof(float) * kNumParams));
@@ -1100,7 +1098,7 @@ int prad_destroy(prad_ctx* c) {
   cudaFree(c->d_cnt);
   cudaFree(c->d_led_emit);
   cudaFree(c->d_led_ll);
-  cudaFree(c->d_partials);
+  cudaFree(c->d_red);
   cudaFree(c->d_sums);
   cudaFree(c->d_mlp);
   cudaFree(c->d_mlp_m);
@@ -1243,7 +1241,7 @@ int prad_angular_histogram(prad_ctx* c, const double axis[3], const double ref[3
 int prad_energy_budget(prad_ctx* c, double* emitted, double* rr_loss, prad_stats* s) {
   if (!c) return fail(c, PRAD_ERR_ARG, "energy_budget: null context");
   CK(c, launch_ledger_reduce(c->d_led_emit, c->d_led_ll, c->cfg.max_particles,
-                             c->d_partials, c->red_blocks, c->d_sums, c->stream));
+                             c->d_red, c->num_sms, c->d_sums, c->stream));
   double sums[2];
   unsigned long long cnt[kNumCounters];
   CK(c, cudaMemcpyAsync(sums, c->d_sums, sizeof(sums), cudaMemcpyDeviceToHost, c->stream));

@@ -316,9 +316,11 @@ cudaError_t launch_ginv_eval(const float* tab, const float* r, float* out, int64
 // words[2i + 1] (the table lookup of the step kernels; push_emit.cu)
 cudaError_t launch_angle_eval(const float* tab, const float* x, const uint32_t* words,
                               float* psi, int64_t n, cudaStream_t s);
-cudaError_t launch_ledger_reduce(const double* a, const double* b, int64_t n,
-                                 double* partials, int nblocks, double* out,
-                                 cudaStream_t s);
+// Exact sums of a[n] and b[n], rounded once, into out[0] and out[1]; scratch
+// of kLedgerScratchBytes on the device (zeroed by the launch itself).
+constexpr size_t kLedgerScratchBytes = 2048;
+cudaError_t launch_ledger_reduce(const double* a, const double* b, int64_t n, void* scratch,
+                                 int num_sms, double* out, cudaStream_t s);
 
 // Run-time specialised kernels (spec.cu): the standard FP32 plane-wave and
 // Yee-grid step kernels compiled by NVRTC with the context's constants as

@@ -296,7 +296,7 @@ def prad_angle_eval(h, x_ptr, words_ptr, out_ptr, n: int) -> None:
 
 
 def prad_ledger_totals_noalloc(emit_ptr, rr_ptr, n: int, out_ptr, stream_ptr=None) -> None:
-    """Kahan totals of two caller-owned device FP64 arrays into a caller-owned
+    """Exact totals (rounded once) of two caller-owned device FP64 arrays into a caller-owned
     device array of 2 doubles, without any device allocation."""
     L = load_library()
     rc = L.prad_ledger_totals_noalloc(emit_ptr, rr_ptr, n, out_ptr, stream_ptr)
