@@ -538,6 +538,7 @@ void fill_common(const prad_ctx* c, StepParams<R>& p, const prad_fields& f) {
     p.tab = c->d_tab32;
   else
     p.tab = c->d_tab64;
+  p.tab32 = c->d_tab32;
   p.px = c->d_ph[0]; p.py = c->d_ph[1]; p.pz = c->d_ph[2];
   p.pnx = c->d_ph[3]; p.pny = c->d_ph[4]; p.pnz = c->d_ph[5];
   p.peps = c->d_ph[6]; p.pw = c->d_ph[7];

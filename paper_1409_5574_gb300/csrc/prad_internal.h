@@ -127,6 +127,7 @@ struct StepParams {
   R inv_dx_lo, inv_dy_lo;      // low parts of 1/dx, 1/dy (float-float)
   // sampling table
   const typename TabOf<R>::T* tab;
+  const float4* tab32;        // the FP32 table in either precision
   R t_scale, x_scale, a;
   uint64_t thr;
   // photons

@@ -241,11 +241,11 @@ __device__ __forceinline__ void sincos_2pi(double v, double* s, double* c) {
 // branches share one log2, so the warp does not diverge.
 // ---------------------------------------------------------------------------
 // STAB: the table is read from a copy in shared memory (stab) instead of
-// through L1 from global memory.
+// through L1 from global memory (gtab).
 template <bool STAB = false>
-__device__ __forceinline__ void sample_x_g(const StepParams<float>& P,
-                                           uint32_t w0, uint32_t w1, float& x,
-                                           float& g, const float4* stab = nullptr) {
+__device__ __forceinline__ void sample_x_g32(const float4* __restrict__ gtab, uint32_t w0,
+                                             uint32_t w1, float& x, float& g,
+                                             const float4* stab = nullptr) {
   const uint64_t W = (static_cast<uint64_t>(w1) << 32) | w0;
   const bool low = W < kThr;
   const uint32_t h = low ? w1 : ~w1;
@@ -269,8 +269,13 @@ __device__ __forceinline__ void sample_x_g(const StepParams<float>& P,
   const float s = u - static_cast<float>(i);
   const int ti = low ? i : kN1 + i;
   float4 c;
-  if constexpr (STAB) c = stab[ti]; else c = __ldg(P.tab + ti);
+  if constexpr (STAB) c = stab[ti]; else c = __ldg(gtab + ti);
   g = fmaf(s, fmaf(s, fmaf(s, c.w, c.z), c.y), c.x);
+}
+template <bool STAB = false>
+__device__ __forceinline__ void sample_x_g(const StepParams<float>& P, uint32_t w0, uint32_t w1,
+                                           float& x, float& g, const float4* stab = nullptr) {
+  sample_x_g32<STAB>(P.tab, w0, w1, x, g, stab);
 }
 
 template <bool STAB = false>
@@ -297,6 +302,22 @@ __device__ __forceinline__ void sample_x_g(const StepParams<double>& P,
   const double s = u - static_cast<double>(i);
   const Coef4d c = P.tab[low ? i : kN1 + i];
   g = fma(s, fma(s, fma(s, c.c3, c.c2), c.c1), c.c0);
+}
+
+// Whether a FP64 trial can matter: false only if its dN is below 1 and below
+// the decision's uniform, so that it neither emits nor counts.  The sampler's
+// logarithm, exponentials and division are about half of the FP64
+// instructions of a step, and few trials emit (a few in a thousand in the
+// constant-field check), so dN is first formed in FP32 from the FP32 table,
+// whose x and g are within 2e-6 of the FP64 ones; the margin of 1e-4 covers
+// that fifty times over.  NaN compares as true.  (10^4 electrons, 1000 steps
+// in a constant field: 8.76 ms without it, 5.10 ms with.)
+__device__ __forceinline__ bool may_emit(const float4* __restrict__ tab32, uint32_t w0,
+                                         uint32_t w1, uint32_t w2, double rate) {
+  float x, g;
+  sample_x_g32(tab32, w0, w1, x, g);
+  const float up = 1.0001f * (static_cast<float>(rate) * (g * __fdividef(1.0f, x)));
+  return !(up < 1.0f && up < unit_uniform<float>(w2));
 }
 
 // ---------------------------------------------------------------------------
@@ -1058,19 +1079,27 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       else
         rnd = philox10_rk<SAMP == PRAD_SAMPLER_TABLE>(make_uint4(pid, step, 0u, P.ensemble), rk);
     }
-    const R Rr = unit_uniform<R>(rnd.z);
     if constexpr (SAMP == PRAD_SAMPLER_TABLE) {
       // 8. Monte Carlo emission: proposal x = P^-1(R'), dN of Eq. (13);
-      //    one trial with the Philox words (w0, w1) and uniform Rd, dN
+      //    one trial with the Philox words (w0, w1, w2), dN
       //    scaled by dn_scale, record weights by wmul, for lanes with part
-      auto trial = [&](uint32_t w0, uint32_t w1, R Rd, R dn_scale, R wmul, bool part,
+      auto trial = [&](uint32_t w0, uint32_t w1, uint32_t w2, R dn_scale, R wmul, bool part,
                        uint32_t j) {
-        R xs, g;
-        sample_x_g<STAB>(P, w0, w1, xs, g, stab);
-        const R dN = P.cn_dt * Om * g * rcp(xs) * dn_scale;
-        const R fl = flr(dN);
-        const R k = fl + ((Rd < dN - fl) ? R(1) : R(0));
-        if (part && dN > R(1)) ++cnt.dn1;
+        R xs = R(1), k = R(0);
+        auto draw = [&] {
+          R g;
+          sample_x_g<STAB>(P, w0, w1, xs, g, stab);
+          const R Rd = unit_uniform<R>(w2);
+          const R dN = P.cn_dt * Om * g * rcp(xs) * dn_scale;
+          const R fl = flr(dN);
+          k = fl + ((Rd < dN - fl) ? R(1) : R(0));
+          if (part && dN > R(1)) ++cnt.dn1;
+        };
+        if constexpr (sizeof(R) == 8) {
+          if (part && may_emit(P.tab32, w0, w1, w2, P.cn_dt * Om * dn_scale)) draw();
+        } else {
+          draw();
+        }
         const bool want = part && k > R(0) && w > R(0);
         // 9. append + emitted-energy ledger; the record is built only when
         //    some lane of the warp emits
@@ -1104,17 +1133,17 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
         }
       };
       if constexpr (!CTRL) {
-        trial(rnd.x, rnd.y, Rr, R(1), R(1), live, 0u);
+        trial(rnd.x, rnd.y, rnd.z, R(1), R(1), live, 0u);
       } else {
         // super-photon control: a particle takes part with probability
         // sel_q (Philox word 3 of trial 0), with weight 1 / sel_q; ntry
         // trials of 1 / ntry of dN each, trial j >= 1 from its own block
         const bool part = live && unit_uniform<R>(rnd.w) < P.sel_q;
-        trial(rnd.x, rnd.y, Rr, P.inv_ntry, P.inv_sel_q, part, 0u);
+        trial(rnd.x, rnd.y, rnd.z, P.inv_ntry, P.inv_sel_q, part, 0u);
         for (int j = 1; j < P.ntry; ++j) {
           const uint4 cj = make_uint4(pid, step, 0x10000u + static_cast<uint32_t>(j), P.ensemble);
           const uint4 rb = philox10_rk(cj, rk);
-          trial(rb.x, rb.y, unit_uniform<R>(rb.z), P.inv_ntry, P.inv_sel_q, part,
+          trial(rb.x, rb.y, rb.z, P.inv_ntry, P.inv_sel_q, part,
                 static_cast<uint32_t>(j));
         }
       }
@@ -1123,6 +1152,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       //     Omega dt (the integral of Eq. (13)'s spectrum), multiplicity as in
       //     the table path; the frequency x = G^-1(r') from the MLP
       const R pm = P.cp_dt * Om;
+      const R Rr = unit_uniform<R>(rnd.z);
       const R fl = flr(pm);
       const R k = fl + ((Rr < pm - fl) ? R(1) : R(0));
       if (live && pm > R(1)) ++cnt.dn1;
