@@ -32,19 +32,21 @@ __device__ __forceinline__ uint4 philox10_mlp(uint4 c, uint32_t k0, uint32_t k1)
 namespace {
 
 constexpr int kTB = 128;  // samples per block (one tile: one sample per thread)
-constexpr int kTZ = kHid + 1;  // padded FP32 rows: column sums without bank conflicts
 
 // Canonical K-major strides (bytes per 8-row group) of the training tiles:
 // K = 64 (delta2 [s][j], W2^T [i][j]) and K = 128 (delta2^T [j][s], h1^T [i][s]).
 constexpr uint32_t kTrSbo64 = (kHid / 8) * 128;
 constexpr uint32_t kTrSbo128 = (kTB / 8) * 128;
 
-// Shared memory of the training kernel (~104 KB: two CTAs per SM).  The
+// Shared memory of the training kernel (~72 KB: three CTAs per SM).  The
 // operand tiles are in the canonical K-major layout of the tensor cores (no
 // swizzle, mlp_tc.cuh).  The forward operands are dead once the forward MMA
-// has completed, and the backward operands take their place.  The dW2 product
-// reads its A operand as 128 rows from d2t: rows 64..127 are h1t's bytes
-// (d2t is followed by h1t), and give TMEM lanes 64..127 that are never read.
+// has completed, and the backward operands take their place; once the
+// backward MMAs have completed, dW2 (on its way to coalesced stores) takes
+// theirs and delta1 that of d2t and h1t.  The dW2 product reads its A operand
+// as 128 rows from d2t: rows 64..127 are h1t's bytes (d2t is followed by
+// h1t), and give TMEM lanes 64..127 that are never read.
+constexpr int kTW = kHid + 1;  // padded rows of dW2 (bank conflicts)
 struct alignas(128) TrainTcSmem {
   union {
     struct {
@@ -55,16 +57,19 @@ struct alignas(128) TrainTcSmem {
       uint16_t d2[kTB * kHid];     // bf16 delta2 [s][j] (delta1, A)
       uint16_t w2t[kHid * kHid];   // BF16 W2^T [i][j] (delta1, B)
     } bwd;
+    float dw2[kHid * kTW];         // dW2 [j][i]
   } u;
-  uint16_t d2t[kHid * kTB];        // bf16 delta2^T [j][s] (dW2, A rows 0..63)
-  uint16_t h1t[kHid * kTB];        // bf16(silu(z1))^T [i][s] (dW2, B)
-  float z1[kTB][kTZ];              // z1, then delta1
+  union {
+    struct {
+      uint16_t d2t[kHid * kTB];    // bf16 delta2^T [j][s] (dW2, A rows 0..63)
+      uint16_t h1t[kHid * kTB];    // bf16(silu(z1))^T [i][s] (dW2, B)
+    } t;
+    float d1[kTB * kHid];          // delta1 [s][i], column i of row s at i ^ (s & 31)
+  } v;
   float wsum[kTB / 32][2 * kHid];  // per-warp sums of dL/dW3 and dL/db2
   float4 w1b1[kHid];               // (BF16 W1 row j, b1 j)
   float w3[kHid];
   float x[kTB][4];                 // features; x[s][3] = 0 valid, -1 padding
-  float tgt[kTB];
-  float wgt[kTB];
   float loss[kTB];
   float dout[kTB];
   float b3;
@@ -73,8 +78,9 @@ struct alignas(128) TrainTcSmem {
 };
 static_assert(offsetof(TrainTcSmem, u.fwd.b2) % 128 == 0 &&
                   offsetof(TrainTcSmem, u.bwd.w2t) % 128 == 0 &&
-                  offsetof(TrainTcSmem, d2t) % 128 == 0 &&
-                  offsetof(TrainTcSmem, h1t) == offsetof(TrainTcSmem, d2t) + kHid * kTB * 2 &&
+                  offsetof(TrainTcSmem, v.t.d2t) % 128 == 0 &&
+                  offsetof(TrainTcSmem, v.t.h1t) ==
+                      offsetof(TrainTcSmem, v.t.d2t) + kHid * kTB * 2 &&
                   offsetof(TrainTcSmem, bar) % 8 == 0,
               "operand and mbarrier alignment; h1t directly after d2t");
 static_assert(tc_off(kTB - 1, kTB - 1, kTrSbo128) < 2 * kHid * kTB &&
@@ -83,22 +89,21 @@ static_assert(tc_off(kTB - 1, kTB - 1, kTrSbo128) < 2 * kHid * kTB &&
                   tc_off(kHid - 1, kHid - 1, kTrSbo64) < kHid * kHid,
               "training tiles stay inside their arrays (dW2's A: d2t and h1t)");
 
-// Warp sums of 64 per-lane values v[0..63] (recursive halving: each round a
+// Warp sums of 32 per-lane values v[0..31] (recursive halving: each round a
 // lane keeps one half of its range and adds its partner's copy of it); lane l
-// ends with the sums of entries 2l and 2l + 1 in v[0] and v[1].
-__device__ __forceinline__ void warp_sum64(float (&v)[kHid], int lane) {
+// ends with the sum of entry l.
+__device__ __forceinline__ float warp_sum32(float (&v)[32], int lane) {
 #pragma unroll
-  for (int r = 0; r < 5; ++r) {
-    const int half = 32 >> r;           // entries kept after this round
-    const int bit = 16 >> r;            // partner lane distance
-    const bool upper = (lane & bit) != 0;
+  for (int half = 16; half; half >>= 1) {
+    const bool upper = (lane & half) != 0;
 #pragma unroll
     for (int k = 0; k < half; ++k) {
       const float keep = upper ? v[k + half] : v[k];
       const float send = upper ? v[k] : v[k + half];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, half);
     }
   }
+  return v[0];
 }
 
 // Training samples: r from a Philox uniform (tag 3), gamma log-uniform in
@@ -167,35 +172,31 @@ __device__ __forceinline__ bool train_wait(TrainTcSmem& S, uint32_t parity) {
 // delta2, bf16(silu(z1)) and W2 in the gradient products, FP32 elsewhere.
 // A tensor-core wait that runs out zeroes the block's partials and sets
 // status bit 2.
-__global__ void __launch_bounds__(kTB, 2)
+//
+// A block is short (one tile) and bound by latency, so what it loads is loaded
+// 16 bytes at a time and early, z1 is formed twice instead of kept (the block
+// then fits three times into an SM), and dW2 goes out in whole lines.  A batch
+// of 65536 samples: 76 us with element-wise images, a 33 KB z1 and two blocks
+// per SM, 36 us so (1.7 rounds of blocks are now 1.1).
+__global__ void __launch_bounds__(kTB, 3)
     k_mlp_train_tc(MlpDev dev, SampleSpec sp, float* __restrict__ partial,
                    float* __restrict__ loss_part, unsigned long long* status) {
   extern __shared__ unsigned char raw[];
   TrainTcSmem& S = *reinterpret_cast<TrainTcSmem*>(
       (reinterpret_cast<uintptr_t>(raw) + 127) & ~static_cast<uintptr_t>(127));
   const int s = threadIdx.x, lane = s & 31, warp = s >> 5;
-  // ---- set-up: the forward weight image, constant columns, mbarrier, TMEM
-  for (int e = s; e < kHid * kTcK2; e += kTB) {  // forward B (unit n, k)
-    const int n = e / kTcK2, k = e - n * kTcK2;
-    float v = 0.0f;
-    if (k < kHid) {
-      v = 0.5f * __bfloat162float(dev.w2[n * kHid + k]);
-    } else if (k < kHid + 2) {
-      const float hb = 0.5f * dev.params[kOffB2 + n];
-      const float hi = __half2float(__float2half_rn(hb));
-      v = k == kHid ? hi : hb - hi;
-    }
-    S.u.fwd.b2[tc_off(n, k, kTcSbo2)] = tc_f16_bits(v);
-  }
-  for (int e = s; e < kTB * 16; e += kTB) {  // forward A columns 64..79: 1 1 0..
-    const int m = e >> 4, k = kHid + (e & 15);
-    S.u.fwd.a2[tc_off(m, k, kTcSbo2)] = k < kHid + 2 ? static_cast<uint16_t>(0x3C00u) : 0;
-  }
+  // ---- set-up: weights on their way, then mbarrier, TMEM and the sample
+  uint4 wq[4];  // W2 row n = e >> 3, units 8 (e & 7) .. + 7, e = s + 128 q
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    wq[q] = *(reinterpret_cast<const uint4*>(dev.w2) + s + kTB * q);
+  float4 w1v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  float w3v = 0.0f, b2v = 0.0f;
   if (s < kHid) {
-    S.w1b1[s] = make_float4(bf16_round(dev.params[kOffW1 + 3 * s]),
-                            bf16_round(dev.params[kOffW1 + 3 * s + 1]),
-                            bf16_round(dev.params[kOffW1 + 3 * s + 2]), dev.params[kOffB1 + s]);
-    S.w3[s] = bf16_round(dev.params[kOffW3 + s]);
+    w1v = make_float4(dev.params[kOffW1 + 3 * s], dev.params[kOffW1 + 3 * s + 1],
+                      dev.params[kOffW1 + 3 * s + 2], dev.params[kOffB1 + s]);
+    w3v = dev.params[kOffW3 + s];
+    b2v = dev.params[kOffB2 + s];
   }
   if (s == 0) {
     S.b3 = dev.params[kOffB3];
@@ -203,37 +204,68 @@ __global__ void __launch_bounds__(kTB, 2)
   }
   __syncwarp();
   if (s < 32) tc_tmem_alloc(&S.tmem, 128);
-  // ---- the block's samples and layer 1 (FP32, BF16 weights)
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * kTB + s;
-  if (idx < sp.n_valid) {
-    make_sample(sp, idx, S.x[s], &S.tgt[s], &S.wgt[s]);
-  } else {  // padding rows contribute nothing
-    S.x[s][0] = S.x[s][1] = S.x[s][2] = 0.0f;
-    S.x[s][3] = -1.0f;
-    S.tgt[s] = 0.0f;
-    S.wgt[s] = 0.0f;
-  }
-  __syncthreads();
-  {
-    const float f0 = S.x[s][0], f1 = S.x[s][1], f2 = S.x[s][2];
-#pragma unroll 4
-    for (int c = 0; c < kHid / 8; ++c) {
-      float z[8];
+  const bool valid = idx < sp.n_valid;
+  float f[4] = {0.0f, 0.0f, 0.0f, -1.0f}, tgt = 0.0f, wgt = 0.0f;
+  if (valid) make_sample(sp, idx, f, &tgt, &wgt);  // (padding rows contribute nothing)
+  S.x[s][0] = f[0];
+  S.x[s][1] = f[1];
+  S.x[s][2] = f[2];
+  S.x[s][3] = f[3];
+  // forward B (unit n, k): halved W2 | split b2
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int j = 8 * c + q;
-        const float4 w = S.w1b1[j];
-        z[q] = fmaf(w.x, f0, fmaf(w.y, f1, fmaf(w.z, f2, w.w)));
-        S.z1[s][j] = z[q];
-        S.h1t[tc_off(j, s, kTrSbo128)] = tc_bf16_bits(silu(z[q]));
-      }
-      uint4 q4;
-      q4.x = silu_f16x2(z[0], z[1]);
-      q4.y = silu_f16x2(z[2], z[3]);
-      q4.z = silu_f16x2(z[4], z[5]);
-      q4.w = silu_f16x2(z[6], z[7]);
-      *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, 8 * c, kTcSbo2)]) = q4;
+  for (int q = 0; q < 4; ++q) {
+    const int e = s + kTB * q, n = e >> 3, c = e & 7;
+    const uint32_t in[4] = {wq[q].x, wq[q].y, wq[q].z, wq[q].w};
+    uint32_t out[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float a = 0.5f * __uint_as_float(in[h] << 16);
+      const float b = 0.5f * __uint_as_float(in[h] & 0xffff0000u);
+      out[h] = static_cast<uint32_t>(tc_f16_bits(a)) |
+               (static_cast<uint32_t>(tc_f16_bits(b)) << 16);
     }
+    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(n, 8 * c, kTcSbo2)]) =
+        make_uint4(out[0], out[1], out[2], out[3]);
+  }
+  if (s < kHid) {
+    S.w1b1[s] = make_float4(bf16_round(w1v.x), bf16_round(w1v.y), bf16_round(w1v.z), w1v.w);
+    S.w3[s] = bf16_round(w3v);
+    const float hb = 0.5f * b2v;
+    const float hi = __half2float(__float2half_rn(hb));
+    const uint32_t pk = static_cast<uint32_t>(tc_f16_bits(hi)) |
+                        (static_cast<uint32_t>(tc_f16_bits(hb - hi)) << 16);
+    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(s, kHid, kTcSbo2)]) = make_uint4(pk, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(s, kHid + 8, kTcSbo2)]) =
+        make_uint4(0u, 0u, 0u, 0u);
+  }
+  // forward A columns 64..79: 1 1 0..
+  *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, kHid, kTcSbo2)]) =
+      make_uint4(0x3C003C00u, 0u, 0u, 0u);
+  *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, kHid + 8, kTcSbo2)]) =
+      make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  // ---- layer 1 (FP32, BF16 weights)
+  const float f0 = f[0], f1 = f[1], f2 = f[2];
+  auto z1 = [&](int j) {
+    const float4 w = S.w1b1[j];
+    return fmaf(w.x, f0, fmaf(w.y, f1, fmaf(w.z, f2, w.w)));
+  };
+#pragma unroll 4
+  for (int c = 0; c < kHid / 8; ++c) {
+    float z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int j = 8 * c + q;
+      z[q] = z1(j);
+      S.v.t.h1t[tc_off(j, s, kTrSbo128)] = tc_bf16_bits(silu(z[q]));
+    }
+    uint4 q4;
+    q4.x = silu_f16x2(z[0], z[1]);
+    q4.y = silu_f16x2(z[2], z[3]);
+    q4.z = silu_f16x2(z[4], z[5]);
+    q4.w = silu_f16x2(z[6], z[7]);
+    *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, 8 * c, kTcSbo2)]) = q4;
   }
   tc_fence_proxy_async();
   tc_fence_before_sync();
@@ -251,68 +283,75 @@ __global__ void __launch_bounds__(kTB, 2)
                  tc_idesc(false, kTB, kHid), k > 0 ? 1u : 0u);
     tc_commit(&S.bar);
   }
+  // W2^T (i, 8 units j) while the MMA runs: i = e & 63, j = 8 (e >> 6) .. + 7
+  uint32_t wt[4][4];
+  {
+    const uint16_t* w2 = reinterpret_cast<const uint16_t*>(dev.w2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int e = s + kTB * q, i = e & (kHid - 1), j = 8 * (e >> 6);
+#pragma unroll
+      for (int h = 0; h < 4; ++h)
+        wt[q][h] = static_cast<uint32_t>(w2[(j + 2 * h) * kHid + i]) |
+                   (static_cast<uint32_t>(w2[(j + 2 * h + 1) * kHid + i]) << 16);
+    }
+  }
   uint32_t pend_par = 0u;  // parity of the MMA group last committed
   bool bad = train_wait(S, 0u);
   if (!bad) {
     // the forward operands are dead: W2^T for the delta1 product takes
     // their place
-    for (int e = s; e < kHid * kHid; e += kTB) {  // W2^T [i][j] = W2[j][i]
-      const int j = e / kHid, i = e - j * kHid;
-      S.u.bwd.w2t[tc_off(i, j, kTrSbo64)] = *reinterpret_cast<const uint16_t*>(dev.w2 + e);
-    }
-    // z2 = 2 c; output o = W3 h2 + b3 with h2 = f16(silu(z2)); loss, dL/do,
-    // delta2 = dL/do W3 silu'(z2)
-    float c2[kHid];
 #pragma unroll
-    for (int half = 0; half < 2; ++half) {
-      uint32_t v[32];
-      tmem_ld_wait_32x32b_x32(lanes + 32 * half, v);
-#pragma unroll
-      for (int q = 0; q < 32; ++q) c2[32 * half + q] = __uint_as_float(v[q]);
+    for (int q = 0; q < 4; ++q) {
+      const int e = s + kTB * q, i = e & (kHid - 1), j = 8 * (e >> 6);
+      *reinterpret_cast<uint4*>(&S.u.bwd.w2t[tc_off(i, j, kTrSbo64)]) =
+          make_uint4(wt[q][0], wt[q][1], wt[q][2], wt[q][3]);
     }
+    // z2 = 2 c; output o = W3 h2 + b3 with h2 = f16(silu(z2)); loss, dL/do
     float o = S.b3;
 #pragma unroll
-    for (int j = 0; j < kHid; j += 2) {
-      const uint32_t hh = silu_half_f16x2(c2[j], c2[j + 1]);
-      const float2 h2 = __half22float2(*reinterpret_cast<const __half2*>(&hh));
-      o = fmaf(S.w3[j], h2.x, o);
-      o = fmaf(S.w3[j + 1], h2.y, o);
-    }
-    const bool valid = S.x[s][3] == 0.0f;
-    const float diff = o - S.tgt[s];
-    const float wg = S.wgt[s];
-    S.loss[s] = valid ? wg * diff * diff : 0.0f;
-    const float dout = valid ? 2.0f * wg * diff / static_cast<float>(sp.n_total) : 0.0f;
-    S.dout[s] = dout;
-    // dL/dW3_j = sum_s dout silu(z2), dL/db2_j = sum_s dout W3_j silu'(z2):
-    // per-warp sums in FP32, then over the warps
-    {
-      float v[kHid];
+    for (int half = 0; half < 2; ++half) {
+      uint32_t c2[32];
+      tmem_ld_wait_32x32b_x32(lanes + 32 * half, c2);
 #pragma unroll
-      for (int j = 0; j < kHid; ++j) v[j] = dout * silu(2.0f * c2[j]);
-      warp_sum64(v, lane);
-      S.wsum[warp][2 * lane] = v[0];
-      S.wsum[warp][2 * lane + 1] = v[1];
-#pragma unroll
-      for (int j = 0; j < kHid; ++j) v[j] = dout * S.w3[j] * silu_grad(2.0f * c2[j]);
-      warp_sum64(v, lane);
-      S.wsum[warp][kHid + 2 * lane] = v[0];
-      S.wsum[warp][kHid + 2 * lane + 1] = v[1];
-    }
-#pragma unroll
-    for (int c = 0; c < kHid / 8; ++c) {
-      uint32_t pk[4];
-#pragma unroll
-      for (int q = 0; q < 8; q += 2) {
-        const int j = 8 * c + q;
-        const float da = dout * S.w3[j] * silu_grad(2.0f * c2[j]);
-        const float db = dout * S.w3[j + 1] * silu_grad(2.0f * c2[j + 1]);
-        pk[q / 2] = pack_bf16x2(da, db);
-        S.d2t[tc_off(j, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] & 0xffffu);
-        S.d2t[tc_off(j + 1, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] >> 16);
+      for (int q = 0; q < 32; q += 2) {
+        const uint32_t hh = silu_half_f16x2(__uint_as_float(c2[q]), __uint_as_float(c2[q + 1]));
+        const float2 h2 = __half22float2(*reinterpret_cast<const __half2*>(&hh));
+        o = fmaf(S.w3[32 * half + q], h2.x, o);
+        o = fmaf(S.w3[32 * half + q + 1], h2.y, o);
       }
-      *reinterpret_cast<uint4*>(&S.u.bwd.d2[tc_off(s, 8 * c, kTrSbo64)]) =
-          make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+    const float diff = o - tgt;
+    S.loss[s] = valid ? wgt * diff * diff : 0.0f;
+    const float dout = valid ? 2.0f * wgt * diff / static_cast<float>(sp.n_total) : 0.0f;
+    S.dout[s] = dout;
+    // delta2 = dL/do W3 silu'(z2); dL/dW3_j = sum_s dout silu(z2), dL/db2_j =
+    // sum_s delta2_j: per-warp sums in FP32, then over the warps
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint32_t c2[32];
+      tmem_ld_wait_32x32b_x32(lanes + 32 * half, c2);
+      float v[32];
+#pragma unroll
+      for (int q = 0; q < 32; ++q)
+        v[q] = dout * S.w3[32 * half + q] * silu_grad(2.0f * __uint_as_float(c2[q]));
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint32_t pk[4];
+#pragma unroll
+        for (int q = 0; q < 8; q += 2) {
+          const int j = 32 * half + 8 * c + q;
+          pk[q / 2] = pack_bf16x2(v[8 * c + q], v[8 * c + q + 1]);
+          S.v.t.d2t[tc_off(j, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] & 0xffffu);
+          S.v.t.d2t[tc_off(j + 1, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] >> 16);
+        }
+        *reinterpret_cast<uint4*>(&S.u.bwd.d2[tc_off(s, 32 * half + 8 * c, kTrSbo64)]) =
+            make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      }
+      S.wsum[warp][kHid + 32 * half + lane] = warp_sum32(v, lane);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) v[q] = dout * silu(2.0f * __uint_as_float(c2[q]));
+      S.wsum[warp][32 * half + lane] = warp_sum32(v, lane);
     }
   }
   // ---- backward products on the tensor cores
@@ -321,7 +360,8 @@ __global__ void __launch_bounds__(kTB, 2)
   __syncthreads();
   tc_fence_after_sync();
   if (!bad && s == 0) {
-    const uint64_t ad = tc_desc(S.d2t, kTcLbo, kTrSbo128), bd = tc_desc(S.h1t, kTcLbo, kTrSbo128);
+    const uint64_t ad = tc_desc(S.v.t.d2t, kTcLbo, kTrSbo128),
+                   bd = tc_desc(S.v.t.h1t, kTcLbo, kTrSbo128);
 #pragma unroll
     for (int k = 0; k < kTB / 16; ++k)
       tc_mma_f16(tmem, ad + k * (kTcKStep >> 4), bd + k * (kTcKStep >> 4),
@@ -346,13 +386,11 @@ __global__ void __launch_bounds__(kTB, 2)
       for (int half = 0; half < 2; ++half) {
         uint32_t v[32];
         tmem_ld_wait_32x32b_x32(lanes + 32 * half, v);
-        // (scalar stores: a block's partials start at a multiple of
-        // kNumParams = 4481 floats, only 4-byte aligned)
 #pragma unroll
-        for (int q = 0; q < 32; ++q) gp[kOffW2 + s * kHid + 32 * half + q] = __uint_as_float(v[q]);
+        for (int q = 0; q < 32; ++q) S.u.dw2[s * kTW + 32 * half + q] = __uint_as_float(v[q]);
       }
     }
-    // delta1 = dh1 silu'(z1), in place of z1
+    // delta1 = dh1 silu'(z1)
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       uint32_t v[32];
@@ -360,7 +398,7 @@ __global__ void __launch_bounds__(kTB, 2)
 #pragma unroll
       for (int q = 0; q < 32; ++q) {
         const int i = 32 * half + q;
-        S.z1[s][i] = __uint_as_float(v[q]) * silu_grad(S.z1[s][i]);
+        S.v.d1[s * kHid + (i ^ lane)] = __uint_as_float(v[q]) * silu_grad(z1(i));
       }
     }
   }
@@ -374,38 +412,41 @@ __global__ void __launch_bounds__(kTB, 2)
       atomicOr(status, 4ull);
     }
   } else {
-    // per-unit sums over the block's samples (FP32)
+#pragma unroll 8
+    for (int e = s; e < kHid * kHid; e += kTB)
+      gp[kOffW2 + e] = S.u.dw2[(e / kHid) * kTW + (e & (kHid - 1))];
+    // per-unit sums over the block's samples (FP32, sample 0 first): unit j,
+    // two of its four sums per thread, beside one of the block's two
+    const int j = s & (kHid - 1);
+    float a = 0.0f, b = 0.0f, t = 0.0f, dsum = 0.0f;
     if (s < kHid) {
-      const int j = s;
-      float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, b1 = 0.0f;
+#pragma unroll 8
       for (int r = 0; r < kTB; ++r) {
-        const float d = S.z1[r][j];
-        a0 = fmaf(d, S.x[r][0], a0);
-        a1 = fmaf(d, S.x[r][1], a1);
-        a2 = fmaf(d, S.x[r][2], a2);
-        b1 += d;
+        const float d = S.v.d1[r * kHid + (j ^ (r & 31))];
+        a = fmaf(d, S.x[r][0], a);
+        b = fmaf(d, S.x[r][1], b);
+        t += S.dout[r];
       }
-      gp[kOffW1 + 3 * j] = a0;
-      gp[kOffW1 + 3 * j + 1] = a1;
-      gp[kOffW1 + 3 * j + 2] = a2;
-      gp[kOffB1 + j] = b1;
-      float dw3 = 0.0f, db2 = 0.0f;
 #pragma unroll
-      for (int w = 0; w < kTB / 32; ++w) {
-        dw3 += S.wsum[w][j];
-        db2 += S.wsum[w][kHid + j];
-      }
-      gp[kOffW3 + j] = dw3;
-      gp[kOffB2 + j] = db2;
-    }
-    if (s == kHid) {
-      float db3 = 0.0f, ls = 0.0f;
+      for (int w = 0; w < kTB / 32; ++w) dsum += S.wsum[w][j];
+      gp[kOffW1 + 3 * j] = a;
+      gp[kOffW1 + 3 * j + 1] = b;
+      gp[kOffW3 + j] = dsum;
+      if (j == 0) gp[kOffB3] = t;
+    } else {
+#pragma unroll 8
       for (int r = 0; r < kTB; ++r) {
-        db3 += S.dout[r];
-        ls += S.loss[r];
+        const float d = S.v.d1[r * kHid + (j ^ (r & 31))];
+        a = fmaf(d, S.x[r][2], a);
+        b += d;
+        t += S.loss[r];
       }
-      gp[kOffB3] = db3;
-      loss_part[blockIdx.x] = ls;
+#pragma unroll
+      for (int w = 0; w < kTB / 32; ++w) dsum += S.wsum[w][kHid + j];
+      gp[kOffW1 + 3 * j + 2] = a;
+      gp[kOffB1 + j] = b;
+      gp[kOffB2 + j] = dsum;
+      if (j == 0) loss_part[blockIdx.x] = t;
     }
   }
   // tear-down: after a timeout, wait (bounded) for the MMAs in flight
@@ -415,23 +456,52 @@ __global__ void __launch_bounds__(kTB, 2)
   if (s < 32) tc_tmem_dealloc(tmem, 128);
 }
 
-// Sum the block partials in a fixed order; optionally Adam-update the FP32
-// master parameters and refresh the BF16 copy of W2.
-__global__ void k_mlp_reduce_adam(const float* __restrict__ partial, int nblocks,
-                                  const float* __restrict__ loss_part, float* __restrict__ grad,
-                                  float* __restrict__ params, float* __restrict__ m,
-                                  float* __restrict__ v, __nv_bfloat16* __restrict__ w2,
-                                  float lr, float b1t, float b2t, int apply,
-                                  float* __restrict__ loss_out, float loss_scale) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == kNumParams) {
-    float ls = 0.0f;
-    for (int b = 0; b < nblocks; ++b) ls += loss_part[b];
-    *loss_out = ls * loss_scale;
-  }
-  if (p >= kNumParams) return;
+// Sum the block partials in a fixed order (block 0 first); optionally
+// Adam-update the FP32 master parameters and refresh the BF16 copy of W2.  A
+// CTA owns 32 parameters (one more slot: the loss): its warps stage rows of 32
+// partials in shared memory with many loads in flight, one warp adds them in
+// order.  (A thread per parameter that reads as it adds waits for 512 loads in
+// turn: 26 us on 18 SMs for the 9.2 MB of a 65536-sample batch, 6 us so.)
+constexpr int kRedParams = 32;
+constexpr int kRedRows = 256;
+constexpr int kRedThreadsAdam = 512;
+__global__ void __launch_bounds__(kRedThreadsAdam)
+    k_mlp_reduce_adam(const float* __restrict__ partial, int nblocks,
+                      const float* __restrict__ loss_part, float* __restrict__ grad,
+                      float* __restrict__ params, float* __restrict__ m, float* __restrict__ v,
+                      __nv_bfloat16* __restrict__ w2, float lr, float b1t, float b2t, int apply,
+                      float* __restrict__ loss_out, float loss_scale) {
+  __shared__ float rows[kRedRows][kRedParams];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int p = blockIdx.x * kRedParams + lane;
+  // one address form for every lane (a branch around the load would keep the
+  // loads from being issued together)
+  const float* src = p < kNumParams ? partial + p : loss_part;
+  const size_t step = p < kNumParams ? kNumParams : 1;
+  constexpr int kWarps = kRedThreadsAdam / 32, kPer = kRedRows / kWarps;
+  float v_in[kPer];  // the rows of the next chunk, in flight while one is added
+  auto fetch = [&](int b0) {
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      v_in[k] = src[static_cast<size_t>(min(b0 + warp + kWarps * k, nblocks - 1)) * step];
+  };
   float gsum = 0.0f;
-  for (int b = 0; b < nblocks; ++b) gsum += partial[static_cast<size_t>(b) * kNumParams + p];
+  fetch(0);
+  for (int b0 = 0; b0 < nblocks; b0 += kRedRows) {
+    const int nb = min(kRedRows, nblocks - b0);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) rows[warp + kWarps * k][lane] = v_in[k];
+    __syncthreads();
+    if (b0 + kRedRows < nblocks) fetch(b0 + kRedRows);
+    if (warp == 0) {
+#pragma unroll 16
+      for (int r = 0; r < nb; ++r) gsum += rows[r][lane];
+    }
+    __syncthreads();
+  }
+  if (warp != 0) return;
+  if (p == kNumParams) *loss_out = gsum * loss_scale;
+  if (p >= kNumParams) return;
   grad[p] = gsum;
   if (!apply) return;
   const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
@@ -607,9 +677,8 @@ cudaError_t launch_mlp_reduce_adam(const float* partial, int nblocks, const floa
                                    __nv_bfloat16* w2, float lr, float b1t, float b2t,
                                    int apply, float* loss_out, float loss_scale,
                                    cudaStream_t s) {
-  const int threads = 256;
-  const int blocks = (kNumParams + 1 + threads - 1) / threads;
-  k_mlp_reduce_adam<<<blocks, threads, 0, s>>>(partial, nblocks, loss_part, grad, params, m,
+  const int blocks = (kNumParams + 1 + kRedParams - 1) / kRedParams;
+  k_mlp_reduce_adam<<<blocks, kRedThreadsAdam, 0, s>>>(partial, nblocks, loss_part, grad, params, m,
                                                 v, w2, lr, b1t, b2t, apply, loss_out,
                                                 loss_scale);
   return cudaGetLastError();
