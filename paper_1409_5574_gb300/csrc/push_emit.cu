@@ -556,13 +556,16 @@ struct PhotonStageRec {
 // The control kernels' layout with the emission's angular spread (CTRL = 2):
 // the fields, plus per record the inputs of its turn, which the flush
 // evaluates for up to 32 records at a time instead of in every warp-step
-// where some lane emits: x, 1/gamma, |u_avg| times the orbit normal, and
-// the two Philox words of psi.
+// where some lane emits: x, 1/gamma, c = u^n x u^(n+1), |u_avg|^2 and the
+// trial (as bits).  The Philox block of psi, the length of the orbit normal
+// and the turn itself cost a warp-step about 100 instructions when the step
+// did them (2^20 electrons at a0 = 500, 100 steps: 1728 us, 1273 us now).
+// FP64 steps scale c themselves, in FP64, and stage -1 for |u_avg|^2.
 struct PhotonStageSpread {
   float f[8][kStage];
   uint32_t pid[kStage];
   uint32_t step[kStage];
-  float ex[7][kStage];  // x, 1/gamma, b_x, b_y, b_z, w0, w1 (words as bits)
+  float ex[7][kStage];  // x, 1/gamma, c_x, c_y, c_z, |u_avg|^2, trial
 };
 
 template <class ST>
@@ -636,7 +639,9 @@ struct PhotonOut {
   const float* ginv;
   double* led_base;
   unsigned long long* fallback;
-  const float* ang;  // angular-spread table (CTRL = 2 kernels)
+  const float* ang;    // angular-spread table (CTRL = 2 kernels)
+  const uint32_t* rk;  // and the round keys and ensemble of psi's draw
+  uint32_t ens;
 };
 
 template <bool PEND = false, class ST>
@@ -654,11 +659,19 @@ __device__ __forceinline__ void flush_stage(ST& st, int fill, const PhotonOut& o
       if constexpr (std::is_same<ST, PhotonStageSpread>::value) {
         // angular spread: u_avg turned by theta = psi / gamma toward b
         float dx = st.f[3][r], dy = st.f[4][r], dz = st.f[5][r];
-        const float bx = st.ex[2][r], by = st.ex[3][r], bz = st.ex[4][r];
+        float bx = st.ex[2][r], by = st.ex[3][r], bz = st.ex[4][r];
+        const float ua2 = st.ex[5][r];
+        if (ua2 >= 0.0f) {  // b = |u_avg| c / |c|
+          const float c2 = bx * bx + by * by + bz * bz;
+          const float fb = c2 > 0.0f ? sqrtf(ua2 / c2) : 0.0f;
+          bx *= fb; by *= fb; bz *= fb;
+        }
         if (bx != 0.0f || by != 0.0f || bz != 0.0f) {
-          const float th = ang_psi<float>(o.ang, st.ex[0][r], __float_as_uint(st.ex[5][r]),
-                                          __float_as_uint(st.ex[6][r])) *
-                           st.ex[1][r];
+          // psi's words: Philox block (pid, step, 0x20000 + trial, ensemble)
+          const uint4 ra = philox10_rk(
+              make_uint4(st.pid[r], st.step[r], 0x20000u + __float_as_uint(st.ex[6][r]), o.ens),
+              o.rk);
+          const float th = ang_psi<float>(o.ang, st.ex[0][r], ra.x, ra.y) * st.ex[1][r];
           float sn, cs;
           sincosf(th, &sn, &cs);
           dx = cs * dx + sn * bx;
@@ -917,7 +930,7 @@ constexpr bool kSharedTab =
 // AOS: the state is P.aos, two vectors per particle (binned Yee launches).
 // STD: the standard configuration (LL kick applied, field form of H_eff,
 // three dimensions, two for the Yee grid) fixed at compile time, so the step
-// tests no mode.
+// tests no mode; with CTRL = 2, one trial and no other control or diagnostic.
 template <typename R, int FIELD, int SAMP, int ONE = 0, int CTRL = 0,
           bool STD = false, bool STAB = false, int PWS = 0, bool AOS = false, class G,
           class ST>
@@ -1029,7 +1042,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       c2 = c2 > R(0) ? c2 : R(0);
       Om = ua2 > R(0) ? R(0.5) * (g0 + g1) * sqr(c2) * rcp(ua2) * P.inv_dtn : R(0);
     }
-    if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE && CTRL) {
+    if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE && CTRL && !STD) {
       if (P.diag & PRAD_DIAG_WIGGLER) {
         // synchrotron (wiggler) regime: Omega tau_EM > 1 with tau_EM the
         // field period the particle sees, 1 / (omega_L |1 - dir beta_x|)
@@ -1114,25 +1127,27 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
                                 static_cast<float>(eps), static_cast<float>(kw)};
           if constexpr (CTRL == 2) {
             // angular spread (Eqs. (5)-(6)): the record carries what its
-            // turn needs (psi's Philox words, block (pid, step, 0x20000 +
-            // trial, ensemble); x; 1/gamma; b = |u_avg| times the orbit
-            // normal u^n x u^(n+1) / |u^n x u^(n+1)|, zero if there is none)
-            // and the flush turns u_avg by theta = psi / gamma toward b
-            const uint4 ra = philox10_rk(make_uint4(pid, step, 0x20000u + j, P.ensemble), rk);
-            const R cx = uy * nuz - uz * nuy, cy = uz * nux - ux * nuz, cz = ux * nuy - uy * nux;
-            const R c2 = cx * cx + cy * cy + cz * cz;
-            const R fb = c2 > R(0) ? sqrt(ua2 / c2) : R(0);
+            // turn needs (c = u^n x u^(n+1), along the orbit normal b /
+            // |u_avg|) and the flush turns u_avg by theta = psi / gamma
+            // toward b
+            R cx = uy * nuz - uz * nuy, cy = uz * nux - ux * nuz, cz = ux * nuy - uy * nux;
+            float len2 = static_cast<float>(ua2);
+            if constexpr (sizeof(R) == 8) {
+              const R c2 = cx * cx + cy * cy + cz * cz;
+              const R fb = c2 > R(0) ? sqrt(ua2 / c2) : R(0);
+              cx *= fb; cy *= fb; cz *= fb;
+              len2 = -1.0f;
+            }
             const float ex[7] = {static_cast<float>(xs), static_cast<float>(iga),
-                                 static_cast<float>(fb * cx), static_cast<float>(fb * cy),
-                                 static_cast<float>(fb * cz), __uint_as_float(ra.x),
-                                 __uint_as_float(ra.y)};
+                                 static_cast<float>(cx), static_cast<float>(cy),
+                                 static_cast<float>(cz), len2, __uint_as_float(j)};
             stage_photon_mask(stage, fill, pout, want, mask, rec, pid, step, ex);
           } else {
             stage_photon_mask(stage, fill, pout, want, mask, rec, pid, step);
           }
         }
       };
-      if constexpr (!CTRL) {
+      if constexpr (!CTRL || STD) {
         trial(rnd.x, rnd.y, rnd.z, R(1), R(1), live, 0u);
       } else {
         // super-photon control: a particle takes part with probability
@@ -1229,6 +1244,8 @@ __device__ __forceinline__ PhotonOut make_pout(const StepParams<R>& P) {
   o.led_base = P.led_base;
   o.fallback = P.counters + kMlpFallback;
   o.ang = P.ang;
+  o.rk = P.rkey;
+  o.ens = P.ensemble;
   return o;
 }
 
@@ -1620,9 +1637,15 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
 
 #ifndef __CUDACC_RTC__
 // The standard-configuration variant (STD) exists for FP32 without control
-// or diagnostics.
+// or diagnostics, or with the angular spread alone.
 template <typename R, int FIELD, int CTRL>
-constexpr bool kHasStd = sizeof(R) == 4 && !CTRL;
+constexpr bool kHasStd = sizeof(R) == 4 && CTRL != 1;
+
+// One trial per step of every particle and no diagnostic but the spread.
+template <typename R>
+bool one_trial(const StepParams<R>& p) {
+  return p.ntry <= 1 && !(p.sel_q < R(1)) && (p.diag & ~PRAD_DIAG_ANGLE_SPREAD) == 0;
+}
 
 // LL kick applied, field-form H_eff, the field's usual dimensions and unit
 // charge (electrons, positrons)
@@ -1653,7 +1676,11 @@ cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cuda
 template <typename R>
 cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int block,
                                    cudaStream_t s) {
-  if (p.ang != nullptr) return launch_tiled_v<R, 2, false>(p, max_work, block, s);
+  if (p.ang != nullptr) {
+    if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
+      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, max_work, block, s);
+    return launch_tiled_v<R, 2, false>(p, max_work, block, s);
+  }
   const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
   if (ctrl) return launch_tiled_v<R, 1, false>(p, max_work, block, s);
   if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
@@ -1665,8 +1692,10 @@ cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int blo
 template <typename R, int FIELD, int SAMP, int PF, int CTRL>
 void launch_k(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
   if constexpr (kHasStd<R, FIELD, CTRL>) {
-    if (std_config(p, FIELD == PRAD_FIELD_YEE2D ? 2 : 3)) {
-      if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE) {
+    if (std_config(p, FIELD == PRAD_FIELD_YEE2D ? 2 : 3) && (CTRL != 2 || one_trial(p))) {
+      // (the spread's kernel reads the signs: with them at compile time the
+      // compiler contracts other products and the results change in the last bit)
+      if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE && CTRL != 2) {
         switch (pw_signs(p)) {
           case 1: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 1><<<grid, block, 0, s>>>(p); return;
           case 2: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 2><<<grid, block, 0, s>>>(p); return;
@@ -1686,7 +1715,7 @@ template <typename R, int FIELD, int SAMP, int PF, int CTRL>
 int occupancy_k(int block, bool std_cfg, int pws) {
   if constexpr (kHasStd<R, FIELD, CTRL>) {
     if (std_cfg) {
-      if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE) {
+      if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE && CTRL != 2) {
         switch (pws) {
           case 1: return occupancy_of(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 1>, block, 0);
           case 2: return occupancy_of(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 2>, block, 0);
@@ -1757,7 +1786,7 @@ cudaError_t launch_field(const StepParams<R>& p, int sampler, int grid, int bloc
 template <typename R, int FIELD, int CTRL>
 int field_occupancy_c(int sampler, int pf, int block, bool std_cfg, int pws) {
   if constexpr (CTRL == 2) {
-    return occupancy_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, 2>(block, false, 0);
+    return occupancy_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, 2>(block, std_cfg, pws);
   } else {
     if (sampler == PRAD_SAMPLER_TABLE) {
       if constexpr (sizeof(R) == 4) {
@@ -1787,9 +1816,10 @@ template <typename R>
 int push_emit_occupancy(const StepParams<R>& p, int field_kind, int sampler, int nsub, int block,
                         bool ctrl) {
   const int pf = nsub == 1 ? (dense_launch(p) ? 2 : 1) : 0;
-  const bool sc = std_config(p, field_kind == PRAD_FIELD_YEE2D ? 2 : 3);
   // the control variant, or its angular-spread form
   const int cv = ctrl ? (p.ang != nullptr ? 2 : 1) : 0;
+  const bool sc = std_config(p, field_kind == PRAD_FIELD_YEE2D ? 2 : 3) &&
+                  (cv != 2 || one_trial(p));
   switch (field_kind) {
     case PRAD_FIELD_CONST:
       return field_occupancy<R, PRAD_FIELD_CONST>(sampler, pf, block, cv, sc, pw_signs(p));
