@@ -346,7 +346,7 @@ int prad_autotune_batch(prad_ctx* ctx, const prad_ensemble* ens, int32_t n_ens,
  * within a cell is not deterministic), and record the tile ranges that
  * push_emit uses to gather from shared-memory field tiles.  push_emit calls it itself every
  * sort_interval steps when sort_interval > 0.  Uses the context's scratch
- * (max_particles x 32 B).  Errors: PRAD_ERR_STATE (fields not YEE2D),
+ * (max_particles x 44 B, FP64 60 B).  Errors: PRAD_ERR_STATE (fields not YEE2D),
  * PRAD_ERR_ARG (null arrays, no pid array, n > max_particles). */
 int prad_sort_by_tile(prad_ctx* ctx, const prad_particles* p, int64_t n);
 

@@ -739,20 +739,51 @@ int ensure_sort(prad_ctx* c, size_t elem) {
   return PRAD_OK;
 }
 
-template <typename R>
-int sort_t(prad_ctx* c, const prad_particles* pp, int64_t n, int chunk = kChunk) {
-  int rc = ensure_sort(c, sizeof(R));
+// The sort of the FP64 path.
+int sort_fp64(prad_ctx* c, const prad_particles* pp, int64_t n, int chunk = kChunk) {
+  int rc = ensure_sort(c, sizeof(double));
   if (rc != PRAD_OK) return rc;
   int ntx, nty;
   const int ntiles = tile_counts(c->fields, &ntx, &nty);
   SortBuffers b = c->sort;
   b.ntiles = ntiles;
-  R* arr[7] = {static_cast<R*>(pp->x), static_cast<R*>(pp->y), static_cast<R*>(pp->z),
-               static_cast<R*>(pp->ux), static_cast<R*>(pp->uy), static_cast<R*>(pp->uz),
-               static_cast<R*>(pp->w)};
+  double* arr[7] = {static_cast<double*>(pp->x),  static_cast<double*>(pp->y),
+                    static_cast<double*>(pp->z),  static_cast<double*>(pp->ux),
+                    static_cast<double*>(pp->uy), static_cast<double*>(pp->uz),
+                    static_cast<double*>(pp->w)};
   const prad_fields& f = c->fields;
-  CK(c, launch_tile_sort<R>(arr, pp->pid, n, b, f.nx, f.ny, f.x0, f.y0, 1.0 / f.dx,
-                            1.0 / f.dy, chunk, c->stream));
+  CK(c, launch_tile_sort<double>(arr, pp->pid, n, b, f.nx, f.ny, f.x0, f.y0, 1.0 / f.dx,
+                                 1.0 / f.dy, chunk, c->stream));
+  return PRAD_OK;
+}
+
+// The FP32 state of p into the tile order of c->bins (the caller holds bin_mu).
+int bin_fp32(prad_ctx* c, const StepParams<float>& p, int chunk) {
+  if (!ensure_bins(c)) return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
+  const prad_fields& f = c->fields;
+  int ntx, nty;
+  BinBuffers b = c->bins;
+  b.ntiles = tile_counts(f, &ntx, &nty);
+  CK(c, launch_tile_bin(p, b, f.x0, f.y0, 1.0 / f.dx, 1.0 / f.dy, chunk, false, c->num_sms,
+                        c->stream));
+  return PRAD_OK;
+}
+
+int sort_fp32(prad_ctx* c, const prad_particles* pp, int64_t n) {
+  std::lock_guard<std::mutex> lk(c->bin_mu);
+  StepParams<float> p{};
+  fill_common<float>(c, p);
+  p.x = static_cast<float*>(pp->x); p.y = static_cast<float*>(pp->y);
+  p.z = static_cast<float*>(pp->z);
+  p.ux = static_cast<float*>(pp->ux); p.uy = static_cast<float*>(pp->uy);
+  p.uz = static_cast<float*>(pp->uz);
+  p.w = static_cast<const float*>(pp->w);
+  p.pid = pp->pid;
+  p.n = n;
+  const int rc = bin_fp32(c, p, kChunk);
+  if (rc != PRAD_OK) return rc;
+  CK(c, launch_tile_unsort(p, c->bins, static_cast<float*>(pp->w), pp->pid, c->num_sms,
+                           c->stream));
   return PRAD_OK;
 }
 
@@ -798,19 +829,19 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   BinBuffers b = c->bins;
   b.ntiles = tile_counts(f, &ntx, &nty);
   p.ntx = ntx;
+  p.aos = b.aos;
   p.work = b.work;
   p.work_count = b.work_count;
   const int chunk = chunk_of(p.n, sub < nsteps ? sub : nsteps, c->num_sms);
   const int mw = static_cast<int>(max_work_items(p.n, b.ntiles, chunk));
   for (int32_t done = 0; done < nsteps;) {
-    CK(c, launch_tile_bin(p, b, f.x0, f.y0, 1.0 / f.dx, 1.0 / f.dy, chunk, c->num_sms,
+    CK(c, launch_tile_bin(p, b, f.x0, f.y0, 1.0 / f.dx, 1.0 / f.dy, chunk, true, c->num_sms,
                           c->stream));
     const int32_t end = done + kBinSteps;
     while (done < nsteps && done < end) {
       const int32_t m = (nsteps - done) < sub ? (nsteps - done) : sub;
       p.t0 = pp->t0 + done;
       p.nsub = m;
-      p.aos = b.aos;
       p.gate = nullptr;
       const SpecFn* spec = nullptr;
       const int rc = spec_for(c, p, true, &spec);
@@ -821,7 +852,6 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
       } else {
         CK(c, launch_push_emit_tiled<float>(p, mw, 256, c->stream));
       }
-      p.aos = nullptr;
       p.gate = b.work_count + 1;
       CK(c, launch_push_emit<float>(p, f.kind, c->cfg.sampler, grid, block, c->stream));
       done += m;
@@ -870,25 +900,36 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
     for (int32_t done = 0; done < nsteps;) {
       const int32_t m = (nsteps - done) < interval ? (nsteps - done) : interval;
       const int chunk = chunk_of(n, m, c->num_sms);
-      int rc = sort_t<R>(c, pp, n, chunk);
-      if (rc != PRAD_OK) return rc;
-      p.work = c->sort.work;
-      p.work_count = c->sort.work_count;
       p.t0 = pp->t0 + done;
       p.nsub = m;
-      const int64_t mw = max_work_items(n, c->sort.ntiles, chunk);
       if constexpr (sizeof(R) == 4) {
+        // the state goes into tile order, is advanced there and comes back in
+        // that order: the caller's particles are reordered
+        std::lock_guard<std::mutex> lk(c->bin_mu);
         const SpecFn* spec = nullptr;
-        rc = spec_for(c, p, true, &spec);
+        int rc = spec_for(c, p, true, &spec);  // (before anything moves)
+        if (rc == PRAD_OK) rc = bin_fp32(c, p, chunk);
         if (rc != PRAD_OK) return rc;
+        p.aos = c->bins.aos;
+        p.work = c->bins.work;
+        p.work_count = c->bins.work_count;
+        const int mw = static_cast<int>(max_work_items(n, ntx * nty, chunk));
         if (spec) {
-          CK(c, spec_launch(spec, p, static_cast<int>(mw), 256, c->stream));
+          CK(c, spec_launch(spec, p, mw, 256, c->stream));
           ++c->spec_launches;
-          done += m;
-          continue;
+        } else {
+          CK(c, launch_push_emit_tiled<R>(p, mw, 256, c->stream));
         }
+        CK(c, launch_tile_unsort(p, c->bins, static_cast<float*>(pp->w), pp->pid, c->num_sms,
+                                 c->stream));
+      } else {
+        const int rc = sort_fp64(c, pp, n, chunk);
+        if (rc != PRAD_OK) return rc;
+        p.work = c->sort.work;
+        p.work_count = c->sort.work_count;
+        const int64_t mw = max_work_items(n, c->sort.ntiles, chunk);
+        CK(c, launch_push_emit_tiled<R>(p, static_cast<int>(mw), 256, c->stream));
       }
-      CK(c, launch_push_emit_tiled<R>(p, static_cast<int>(mw), 256, c->stream));
       done += m;
     }
     return PRAD_OK;
@@ -1164,8 +1205,8 @@ int prad_sort_by_tile(prad_ctx* c, const prad_particles* p, int64_t n) {
   int rc = check_sort_args(c, p, n);
   if (rc != PRAD_OK) return rc;
   if (n == 0) return PRAD_OK;
-  if (c->cfg.precision == PRAD_FP32) return sort_t<float>(c, p, n);
-  return sort_t<double>(c, p, n);
+  if (c->cfg.precision == PRAD_FP32) return sort_fp32(c, p, n);
+  return sort_fp64(c, p, n);
 }
 
 int prad_get_photons(prad_ctx* c, prad_photons* out, int64_t cap, int64_t* n_out,

@@ -152,10 +152,9 @@ struct StepParams {
   const int4* work;           // (tile, first, end, 0) per work item
   const unsigned int* work_count;
   int32_t ntx;                // tiles along x
-  // binned Yee gather (particles stay in the caller's order): the state in
-  // tile and cell order, two vectors per particle, (x, y, z, u_x) and
-  // (u_y, u_z, w, id as bits); the plain kernel that stands behind it runs
-  // only where *gate is not 0
+  // binned Yee gather: the FP32 state in tile and cell order, two vectors per
+  // particle, (x, y, z, u_x) and (u_y, u_z, w, id as bits); a plain kernel
+  // that stands behind it runs only where *gate is not 0
   float4* aos;
   const unsigned int* gate;
   // Philox4x32-10 round keys of (key0, key1) (philox_round_keys), read
@@ -250,7 +249,6 @@ cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
                                 R* x_out, R* g_out, int64_t n, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
                           uint32_t* out, int64_t n, cudaStream_t s);
-// (p.aos: the binned form)
 template <typename R>
 cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int block,
                                    cudaStream_t s);
@@ -260,9 +258,14 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
                              double inv_dy, int chunk, cudaStream_t s);
 // The state of the p.n particles of p into b.aos in the order of their tiles
 // and cells, and the work list (chunks of at most `chunk` particles of one
-// tile); launch_tile_unbin writes it back to where it came from.
+// tile); gate: sparse particles leave that to the plain kernel.
+// launch_tile_unbin writes the state back to where it came from,
+// launch_tile_unsort in its new order, with the weights and ids.
 cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
-                            double inv_dx, double inv_dy, int chunk, int num_sms, cudaStream_t s);
+                            double inv_dx, double inv_dy, int chunk, bool gate, int num_sms,
+                            cudaStream_t s);
+cudaError_t launch_tile_unsort(const StepParams<float>& p, const BinBuffers& b, float* w,
+                               uint32_t* pid, int num_sms, cudaStream_t s);
 cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, int num_sms,
                               cudaStream_t s);
 size_t mlp_train_smem_bytes();
@@ -326,7 +329,7 @@ cudaError_t launch_ledger_reduce(const double* a, const double* b, int64_t n, vo
 // Run-time specialised kernels (spec.cu): the standard FP32 plane-wave and
 // Yee-grid step kernels compiled by NVRTC with the context's constants as
 // literals.  A variant names the kernel (k_push_emit, or k_push_emit_tiled
-// when tiled, 2 its binned form), field model, sampler, prefetch mode and plane-wave signs.
+// when tiled), field model, sampler, prefetch mode and plane-wave signs.
 // spec_get returns its kernel for these parameters' constants, compiling it
 // on first use (an error, with a message in msg, when NVRTC or the driver
 // cannot provide it).

@@ -1575,14 +1575,15 @@ int batch_max_blocks_per_sm(int block, int sampler, bool ctrl, bool std_cfg) {
 // (+ halo, periodic) in shared memory with coalesced row loads, then runs the
 // same per-particle path with the shared-memory gather.
 // ---------------------------------------------------------------------------
-// AOS: the binned form, for particles kept in another order (P.aos).
-template <typename R, int CTRL, bool STD = false, bool AOS = false>
+// FP32: the state is the binned copy (P.aos).
+template <typename R, int CTRL, bool STD = false>
 __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> P_arg) {
 #ifdef PRAD_SPEC
   const StepParams<R> P = spec_params(P_arg);
 #else
   const StepParams<R>& P = P_arg;
 #endif
+  constexpr bool kAos = sizeof(R) == 4;
   if (blockIdx.x >= *P.work_count) return;
   extern __shared__ __align__(16) float tile_sm[];
   using Stage = typename std::conditional<CTRL == 2, PhotonStageSpread, PhotonStageSoA>::type;
@@ -1624,11 +1625,11 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   for (int64_t base = wk.y; base < wk.z; base += blockDim.x) {
     const int64_t i = base + threadIdx.x;
     PState<R> st;
-    if constexpr (AOS)
+    if constexpr (kAos)
       load_aos(P, i, i < wk.z, st);
     else
       load_state(P, i, i < wk.z, st);
-    advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, AOS>(
+    advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, kAos>(
         P, P.rkey, gat, i, st, stage, fill, pout, cnt);
   }
   if (fill > 0) flush_stage(stage, fill, pout);
@@ -1655,22 +1656,15 @@ bool std_config(const StepParams<R>& p, int dims) {
          p.abs_q == R(1);
 }
 
-template <typename R, int CTRL, bool STD, bool AOS>
-cudaError_t launch_tiled_a(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
+template <typename R, int CTRL, bool STD>
+cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
   // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
-  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD, AOS>,
+  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kTileSmemBytes);
   if (e != cudaSuccess) return e;
-  k_push_emit_tiled<R, CTRL, STD, AOS><<<max_work, block, kTileSmemBytes, s>>>(p);
+  k_push_emit_tiled<R, CTRL, STD><<<max_work, block, kTileSmemBytes, s>>>(p);
   return cudaGetLastError();
-}
-
-template <typename R, int CTRL, bool STD>
-cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
-  if constexpr (sizeof(R) == 4)
-    if (p.aos) return launch_tiled_a<R, CTRL, STD, true>(p, max_work, block, s);
-  return launch_tiled_a<R, CTRL, STD, false>(p, max_work, block, s);
 }
 
 template <typename R>
@@ -1836,7 +1830,7 @@ bool push_emit_spec_variant(const StepParams<float>& p, int field_kind, int samp
   if (ctrl) return false;
   v->field = field_kind;
   v->samp = sampler;
-  v->tiled = tiled ? (p.aos ? 2 : 1) : 0;
+  v->tiled = tiled ? 1 : 0;
   v->pf = 0;
   v->pws = 0;
   if (tiled) return field_kind == PRAD_FIELD_YEE2D && sampler == PRAD_SAMPLER_TABLE &&

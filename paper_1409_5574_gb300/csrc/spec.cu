@@ -286,8 +286,7 @@ cudaError_t spec_get_impl(SpecCache* c, int device, const StepParams<float>& p,
   }
   char name[160];
   if (v.tiled)
-    std::snprintf(name, sizeof(name), "prad::k_push_emit_tiled<float, false, true, %s>",
-                  v.tiled == 2 ? "true" : "false");
+    std::snprintf(name, sizeof(name), "prad::k_push_emit_tiled<float, false, true>");
   else
     std::snprintf(name, sizeof(name), "prad::k_push_emit<float, %d, %d, %d, false, true, %d>",
                   v.field, v.samp, v.pf, v.pws);

@@ -1,7 +1,5 @@
 // Counting sort of particles by the 32 x 32-cell tile of the 2D Yee grid that
-// holds them (histogram -> exclusive scan -> scatter into a scratch copy), then
-// by cell inside each tile (one block per tile, scattering back into the
-// caller's arrays), and the work list of the tile-staged gather kernel: one
+// holds them and by cell inside each tile, and the work list of the tile-staged gather kernel: one
 // item per chunk of at most kChunk particles of one tile.  In cell order the
 // lanes of a warp read the same or neighbouring stencil values of the staged
 // tile (broadcasts instead of shared-memory bank conflicts).  Particles keep
@@ -145,7 +143,7 @@ __global__ void __launch_bounds__(kScanThreads)
       starts[ntiles] = ia;
       const bool none = sparse != 0u && ia < static_cast<uint64_t>(sparse) * tiles;
       work_count[0] = none ? 0u : ib;
-      if (sparse != 0u) work_count[1] = none ? 1u : 0u;
+      work_count[1] = none ? 1u : 0u;
     }
   }
   __syncthreads();
@@ -256,9 +254,10 @@ __global__ void __launch_bounds__(kCellThreads)
 }
 
 // ---------------------------------------------------------------------------
-// Binning: a copy of the state in the same order (tile, then cell), for
-// particles that stay where the caller keeps them.  The caller's arrays are
-// only ever streamed; the scattered side is the copy, whose particles are
+// FP32, binning: a copy of the state in that order, on which the tile-staged
+// kernel runs.  It goes back to where it came from (particles that stay in
+// the caller's order) or, for the sorted path, in its own order, both streams
+// of whole lines.  The caller's arrays are only ever streamed; the scattered side is the copy, whose particles are
 // one 32-byte sector each.  (Gathering the seven arrays through an index in
 // the push itself cost 0.25 ns per particle and launch on 8M particles in
 // random order; now 2^21 particles in random order take 13 us to count, 6 to
@@ -380,6 +379,7 @@ __global__ void __launch_bounds__(kBinThreads)
   s_cnt[tid] = 0u;
   s_cnt[tid + kBinThreads] = 0u;
   __syncthreads();
+#pragma unroll 4
   for (unsigned int k = a + tid; k < b; k += kBinThreads) atomicAdd(s_cnt + keys[k].y, 1u);
   __syncthreads();
   // exclusive scan, thread tid holding cells 2 tid and 2 tid + 1
@@ -396,6 +396,7 @@ __global__ void __launch_bounds__(kBinThreads)
   s_cnt[2 * tid] = e0;
   s_cnt[2 * tid + 1] = e0 + c0;
   __syncthreads();
+#pragma unroll 4
   for (unsigned int k = a + tid; k < b; k += kBinThreads) {
     const uint2 q = keys[k];
     slot[q.x] = a + atomicAdd(s_cnt + q.y, 1u);
@@ -434,6 +435,25 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// The copy back in its own order: the caller's particles reordered.
+__global__ void __launch_bounds__(256)
+    k_bin_unsort(const StepParams<float> P, const float4* __restrict__ aos,
+                 float* __restrict__ w, uint32_t* __restrict__ pid) {
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < P.n;
+       i += stride) {
+    const float4 a = aos[2 * i], b = aos[2 * i + 1];
+    P.x[i] = a.x;
+    P.y[i] = a.y;
+    if (P.z) P.z[i] = a.z;
+    P.ux[i] = a.w;
+    P.uy[i] = b.x;
+    P.uz[i] = b.y;
+    w[i] = b.z;
+    pid[i] = __float_as_uint(b.w);
+  }
+}
+
 int stream_grid(int64_t n, int num_sms) {
   const int64_t want = (n + 255) / 256, cap = 8 * static_cast<int64_t>(num_sms);
   return static_cast<int>(want < cap ? want : cap);
@@ -442,7 +462,7 @@ int stream_grid(int64_t n, int num_sms) {
 }  // namespace
 
 cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
-                            double inv_dx, double inv_dy, int chunk, int num_sms,
+                            double inv_dx, double inv_dy, int chunk, bool gate, int num_sms,
                             cudaStream_t s) {
   const int64_t n = p.n;
   const float *x = p.x, *y = p.y;
@@ -479,7 +499,7 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, dou
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_tile_scan<<<1, kScanThreads, 0, s>>>(b.counts, b.ntiles, b.starts, b.cursor, b.work,
                                           b.work_count, static_cast<unsigned int>(chunk),
-                                          kBinSparse);
+                                          gate ? kBinSparse : 0u);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (sm)
     k_bin_scatter<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.cursor, b.keys);
@@ -498,6 +518,13 @@ cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, i
   return cudaGetLastError();
 }
 
+cudaError_t launch_tile_unsort(const StepParams<float>& p, const BinBuffers& b, float* w,
+                               uint32_t* pid, int num_sms, cudaStream_t s) {
+  k_bin_unsort<<<stream_grid(p.n, num_sms), 256, 0, s>>>(p, b.aos, w, pid);
+  return cudaGetLastError();
+}
+
+// The FP64 sort (its records are too long for the sectors the binning moves).
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,
                              int nx, int ny, double x0, double y0, double inv_dx,
@@ -528,9 +555,6 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
   return cudaGetLastError();
 }
 
-template cudaError_t launch_tile_sort<float>(float* [7], uint32_t*, int64_t, const SortBuffers&,
-                                             int, int, double, double, double, double, int,
-                                             cudaStream_t);
 template cudaError_t launch_tile_sort<double>(double* [7], uint32_t*, int64_t,
                                               const SortBuffers&, int, int, double, double,
                                               double, double, int, cudaStream_t);
