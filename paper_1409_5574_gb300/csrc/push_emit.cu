@@ -210,6 +210,19 @@ __device__ __forceinline__ double sqr(double v) { return sqrt(v); }
 // non-finite argument belongs to a frozen particle, which is never stored)
 __device__ __forceinline__ float sqr_pos(float v) { return v * rsqrtf(v); }
 __device__ __forceinline__ double sqr_pos(double v) { return sqrt(v); }
+// v > 0 ? v : 0, and a > b for a, b >= 0.  A FP64 compare is an instruction of
+// the FP64 pipe, which holds a warp for 64 clocks on GB300 however few of its
+// lanes are active; the bits of nonnegative doubles compare as integers.
+// (v below 2^-1042 counts as 0; a NaN a is not above.)
+__device__ __forceinline__ float positive_part(float v) { return v > 0.0f ? v : 0.0f; }
+__device__ __forceinline__ double positive_part(double v) {
+  return static_cast<uint32_t>(__double2hiint(v)) - 1u < 0x7ff00000u ? v : 0.0;
+}
+__device__ __forceinline__ bool above(float a, float b) { return a > b; }
+__device__ __forceinline__ bool above(double a, double b) {
+  const long long x = __double_as_longlong(a);
+  return x > __double_as_longlong(b) && x <= 0x7ff0000000000000ll;
+}
 __device__ __forceinline__ float flr(float v) { return floorf(v); }
 __device__ __forceinline__ double flr(double v) { return floor(v); }
 __device__ __forceinline__ float rnd_int(float v) { return rintf(v); }
@@ -287,10 +300,11 @@ __device__ __forceinline__ void sample_x_g(const StepParams<double>& P,
   const bool low = W < kThr;
   double u;
   if (low) {
+    // two roots: a quarter of the FP64 instructions of a logarithm and two
+    // exponentials, and x and t to a unit or two in the last place
     const double Rp = fma(static_cast<double>(W), 0x1p-64, 0x1p-65);
-    const double L = log2(Rp);
-    const double t = exp2(0.25 * L);
-    x = exp2(0.75 * L);
+    const double t = sqrt(sqrt(Rp));
+    x = t * t * t;
     u = t * kTScale;
   } else {
     const double om = fma(static_cast<double>(~W), 0x1p-64, 0x1p-65);
@@ -980,6 +994,11 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
   const int rr_mode = STD ? PRAD_RR_APPLY : P.rr_mode;
   const int heff_form = STD ? PRAD_HEFF_FIELD : P.heff_form;
   const int dims = STD ? (FIELD == PRAD_FIELD_YEE2D ? 2 : 3) : P.dims;
+  // a pure magnetic field in FP64, whose instructions are what the step waits
+  // for (false at compile time elsewhere)
+  bool no_e = false;
+  if constexpr (sizeof(R) == 8 && FIELD == PRAD_FIELD_CONST)
+    no_e = P.E[0] == R(0) && P.E[1] == R(0) && P.E[2] == R(0);
   for (int s = 0; s < nsub; ++s) {
     const uint32_t step = static_cast<uint32_t>(P.t0 + s);
     // 1. field at x^n, t^n
@@ -1005,6 +1024,19 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       nux = umx + (vy * sz - vz * sy);
       nuy = umy - vx * sz + hq * f.Ey;
       nuz = umz + vx * sy + hq * f.Ez;
+    } else if (no_e) {
+      // (E = 0 in FP64: the same push, its zero terms left out)
+      const R umx = ux, umy = uy, umz = uz;
+      const R igm = rsq(R(1) + umx * umx + umy * umy + umz * umz);
+      const R tx = hq * f.Bx * igm, ty = hq * f.By * igm, tz = hq * f.Bz * igm;
+      const R sf = R(2) * rcp(R(1) + tx * tx + ty * ty + tz * tz);
+      const R sx = sf * tx, sy = sf * ty, sz = sf * tz;
+      const R vx = umx + (umy * tz - umz * ty);
+      const R vy = umy + (umz * tx - umx * tz);
+      const R vz = umz + (umx * ty - umy * tx);
+      nux = umx + (vy * sz - vz * sy);
+      nuy = umy + (vz * sx - vx * sz);
+      nuz = umz + (vx * sy - vy * sx);
     } else {
       const R umx = ux + hq * f.Ex, umy = uy + hq * f.Ey, umz = uz + hq * f.Ez;
       const R igm = rsq(R(1) + umx * umx + umy * umy + umz * umz);
@@ -1033,14 +1065,21 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
         fy = f.Ey - bx * f.Bz;
         fz = f.Ez + bx * f.By;
         eb = f.Ey * by + f.Ez * bz;
+      } else if (no_e) {
+        fx = by * f.Bz - bz * f.By;
+        fy = bz * f.Bx - bx * f.Bz;
+        fz = bx * f.By - by * f.Bx;
+        eb = R(0);
       } else {
         fx = f.Ex + (by * f.Bz - bz * f.By);
         fy = f.Ey + (bz * f.Bx - bx * f.Bz);
         fz = f.Ez + (bx * f.By - by * f.Bx);
         eb = f.Ex * bx + f.Ey * by + f.Ez * bz;
       }
-      const R h2 = fx * fx + fy * fy + fz * fz - eb * eb;
-      Om = (STD ? R(1) : P.abs_q) * sqr(h2 > R(0) ? h2 : R(0));
+      R h2 = fx * fx + fy * fy + fz * fz;
+      if (!no_e) h2 = fx * fx + fy * fy + fz * fz - eb * eb;
+      // (the charge is +1 or -1: a factor 1, left out of the FP64 steps)
+      Om = (STD || sizeof(R) == 8 ? R(1) : P.abs_q) * sqr(positive_part(h2));
     } else {  // Eq. (9), gamma = mean of the end-point Lorentz factors
       const R dx_ = nux - ux, dy_ = nuy - uy, dz_ = nuz - uz;
       const R dp2 = dx_ * dx_ + dy_ * dy_ + dz_ * dz_;
@@ -1059,7 +1098,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
         if (live && Om < seen) ++cnt.wig;
       }
     }
-    if (Om * P.dtn > ga) {
+    if (above(Om * P.dtn, ga)) {
       Om = ga * P.inv_dtn;
       if (live) ++cnt.clamp;
     }
@@ -1067,7 +1106,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
     //    tested as 1.5 chi > 1.5 on the product epsc is formed from
     const R e1 = P.eps_r15 * Om * ga;
     const R epsc = e1 * ga;
-    if (live && e1 > R(1.5)) ++cnt.chi;
+    if (live && above(e1, R(1.5))) ++cnt.chi;
     // 6. Landau-Lifshitz loss (Eq. (4)): ledger and optional kick
     const R om2 = Om * Om;
     if (rr_mode >= PRAD_RR_LEDGER) ll.add(w * P.ll_coef * om2 * ua2);
@@ -1742,6 +1781,19 @@ bool dense_launch(const StepParams<R>& p) {
          (p.rr_mode < PRAD_RR_LEDGER || p.led_ll != nullptr);
 }
 
+// Whether a one-step launch runs the prefetching kernel: on analytic fields,
+// where the state's stream is what it waits for (2^22 particles 66.5 against
+// 93.1 us; alike below 2^17).  On the Yee grid the gather is, and the plain
+// kernel keeps more of it in flight and leaves L1 to it (2^16 particles 15.8
+// against 19.1 us, 2^22 562 against 716).
+// (A fused launch reads its state once; prefetching would cost it registers.)
+template <typename R, int FIELD>
+constexpr bool kHasStream = sizeof(R) == 4 && FIELD != PRAD_FIELD_YEE2D;
+template <typename R>
+bool stream_launch(const StepParams<R>&, int field_kind, int nsub) {
+  return sizeof(R) == 4 && nsub == 1 && field_kind != PRAD_FIELD_YEE2D;
+}
+
 template <typename R, int FIELD, int CTRL>
 cudaError_t launch_field_c(const StepParams<R>& p, int sampler, int grid, int block,
                            cudaStream_t s) {
@@ -1751,19 +1803,16 @@ cudaError_t launch_field_c(const StepParams<R>& p, int sampler, int grid, int bl
     return cudaGetLastError();
   } else {
     if (sampler == PRAD_SAMPLER_TABLE) {
-      // prefetching pays when the state streams through HBM (one step per
-      // launch); for long fused launches it only costs registers
-      bool pf = false;
-      if constexpr (sizeof(R) == 4) pf = p.nsub == 1;
-      if constexpr (sizeof(R) == 4) {
-        if (pf) {
+      if constexpr (kHasStream<R, FIELD>) {
+        if (stream_launch(p, FIELD, p.nsub)) {
           if (dense_launch(p))
             launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 2, CTRL>(p, grid, block, s);
           else
             launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 1, CTRL>(p, grid, block, s);
+          return cudaGetLastError();
         }
       }
-      if (!pf) launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, CTRL>(p, grid, block, s);
+      launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, CTRL>(p, grid, block, s);
       return cudaGetLastError();
     }
     if constexpr (sizeof(R) == 4) {
@@ -1792,7 +1841,7 @@ int field_occupancy_c(int sampler, int pf, int block, bool std_cfg, int pws) {
     return occupancy_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, 2>(block, std_cfg, pws);
   } else {
     if (sampler == PRAD_SAMPLER_TABLE) {
-      if constexpr (sizeof(R) == 4) {
+      if constexpr (kHasStream<R, FIELD>) {
         if (pf == 2) return occupancy_k<R, FIELD, PRAD_SAMPLER_TABLE, 2, CTRL>(block, std_cfg, pws);
         if (pf == 1) return occupancy_k<R, FIELD, PRAD_SAMPLER_TABLE, 1, CTRL>(block, std_cfg, pws);
       }
@@ -1818,7 +1867,7 @@ int field_occupancy(int sampler, int pf, int block, int ctrl, bool std_cfg, int 
 template <typename R>
 int push_emit_occupancy(const StepParams<R>& p, int field_kind, int sampler, int nsub, int block,
                         bool ctrl) {
-  const int pf = nsub == 1 ? (dense_launch(p) ? 2 : 1) : 0;
+  const int pf = stream_launch(p, field_kind, nsub) ? (dense_launch(p) ? 2 : 1) : 0;
   // the control variant, or its angular-spread form
   const int cv = ctrl ? (p.ang != nullptr ? 2 : 1) : 0;
   const bool sc = std_config(p, field_kind == PRAD_FIELD_YEE2D ? 2 : 3) &&
@@ -1853,7 +1902,8 @@ bool push_emit_spec_variant(const StepParams<float>& p, int field_kind, int samp
     return false;
   }
   // (the learned samplers have no prefetching variant)
-  v->pf = sampler != PRAD_SAMPLER_TABLE ? 0 : p.nsub == 1 ? (dense_launch(p) ? 2 : 1) : 0;
+  v->pf = sampler != PRAD_SAMPLER_TABLE || !stream_launch(p, field_kind, p.nsub) ? 0
+                                                                    : dense_launch(p) ? 2 : 1;
   return true;
 }
 template int push_emit_occupancy<double>(const StepParams<double>&, int, int, int, int, bool);
