@@ -218,6 +218,21 @@ __device__ __forceinline__ float positive_part(float v) { return v > 0.0f ? v : 
 __device__ __forceinline__ double positive_part(double v) {
   return static_cast<uint32_t>(__double2hiint(v)) - 1u < 0x7ff00000u ? v : 0.0;
 }
+// A FP64 value >= 0 cut to FP32 by its bits (off by less than 2^-23 of it);
+// NaN outside FP32's normal range.  maybe_above: false only if such values
+// are not above each other; NaN says maybe.  FP32 steps compare directly.
+__device__ __forceinline__ float trunc32(double v) {
+  const uint32_t hi = static_cast<uint32_t>(__double2hiint(v));
+  const uint32_t lo = static_cast<uint32_t>(__double2loint(v));
+  return __uint_as_float(hi - (897u << 20) < (253u << 20)
+                             ? __funnelshift_l(lo, hi - (896u << 20), 3)
+                             : 0x7fffffffu);
+}
+__device__ __forceinline__ float trunc32(float v) { return v; }
+template <typename R>
+__device__ __forceinline__ bool maybe_above(float a, float b) {
+  return sizeof(R) == 4 || !(a < b);
+}
 __device__ __forceinline__ bool above(float a, float b) { return a > b; }
 __device__ __forceinline__ bool above(double a, double b) {
   const long long x = __double_as_longlong(a);
@@ -325,12 +340,14 @@ __device__ __forceinline__ void sample_x_g(const StepParams<double>& P,
 // constant-field check), so dN is first formed in FP32 from the FP32 table,
 // whose x and g are within 2e-6 of the FP64 ones; the margin of 1e-4 covers
 // that fifty times over.  NaN compares as true.  (10^4 electrons, 1000 steps
-// in a constant field: 8.76 ms without it, 5.10 ms with.)
+// in a constant field: 8.76 ms without it, 5.10 ms with; 4.05 with the FP64
+// instructions left out elsewhere in the step, 104 per warp-step at 64 clocks
+// each.)
 __device__ __forceinline__ bool may_emit(const float4* __restrict__ tab32, uint32_t w0,
-                                         uint32_t w1, uint32_t w2, double rate) {
+                                         uint32_t w1, uint32_t w2, float rate) {
   float x, g;
   sample_x_g32(tab32, w0, w1, x, g);
-  const float up = 1.0001f * (static_cast<float>(rate) * (g * __fdividef(1.0f, x)));
+  const float up = 1.0001f * (rate * (g * __fdividef(1.0f, x)));
   return !(up < 1.0f && up < unit_uniform<float>(w2));
 }
 
@@ -997,8 +1014,13 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
   // a pure magnetic field in FP64, whose instructions are what the step waits
   // for (false at compile time elsewhere)
   bool no_e = false;
+  R ig_last = R(0);
   if constexpr (sizeof(R) == 8 && FIELD == PRAD_FIELD_CONST)
     no_e = P.E[0] == R(0) && P.E[1] == R(0) && P.E[2] == R(0);
+  // FP32 views for the tests that FP32 can answer
+  const float dtn32 = static_cast<float>(P.dtn), eps32 = static_cast<float>(P.eps_r15),
+              cn32 = static_cast<float>(P.cn_dt);
+  (void)dtn32; (void)eps32; (void)cn32;
   for (int s = 0; s < nsub; ++s) {
     const uint32_t step = static_cast<uint32_t>(P.t0 + s);
     // 1. field at x^n, t^n
@@ -1025,9 +1047,14 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       nuy = umy - vx * sz + hq * f.Ey;
       nuz = umz + vx * sy + hq * f.Ez;
     } else if (no_e) {
-      // (E = 0 in FP64: the same push, its zero terms left out)
+      // (E = 0 in FP64: the same push, its zero terms left out; without the
+      // LL kick 1/gamma is the previous step's, from the same momentum)
       const R umx = ux, umy = uy, umz = uz;
-      const R igm = rsq(R(1) + umx * umx + umy * umy + umz * umz);
+      if (s == 0 || rr_mode == PRAD_RR_APPLY) {
+        const R m2 = umx * umx + umy * umy + umz * umz;
+        ig_last = rsq(R(1) + m2);
+      }
+      const R igm = ig_last;
       const R tx = hq * f.Bx * igm, ty = hq * f.By * igm, tz = hq * f.Bz * igm;
       const R sf = R(2) * rcp(R(1) + tx * tx + ty * ty + tz * tz);
       const R sx = sf * tx, sy = sf * ty, sz = sf * tz;
@@ -1052,13 +1079,23 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
     }
     // 3. mean momentum of the step
     const R ax = R(0.5) * (ux + nux), ay = R(0.5) * (uy + nuy), az = R(0.5) * (uz + nuz);
-    const R ua2 = ax * ax + ay * ay + az * az;
+    R ua2 = ax * ax + ay * ay + az * az;
+    if constexpr (sizeof(R) == 8) {
+      // from the sums, whose halves are exact: the same value, and the halves
+      // are only formed for a record
+      const R sx = ux + nux, sy = uy + nuy, sz = uz + nuz;
+      ua2 = R(0.25) * (sx * sx + sy * sy + sz * sz);
+    }
     const R iga = rsq(R(1) + ua2);
     const R ga = (R(1) + ua2) * iga;
     // 4. effective field, limited by dp_perp/p <= 1 (Omega dt <= gamma)
     R Om;
     if (heff_form == PRAD_HEFF_FIELD) {
-      const R bx = ax * iga, by = ay * iga, bz = az * iga;
+      R bx = ax * iga, by = ay * iga, bz = az * iga;
+      if constexpr (sizeof(R) == 8) {
+        const R h = R(0.5) * iga;
+        bx = (ux + nux) * h; by = (uy + nuy) * h; bz = (uz + nuz) * h;
+      }
       R fx, fy, fz, eb;
       if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE) {
         fx = by * f.Bz - bz * f.By;
@@ -1098,15 +1135,18 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
         if (live && Om < seen) ++cnt.wig;
       }
     }
-    if (above(Om * P.dtn, ga)) {
+    float om32 = trunc32(Om);
+    const float ga32 = trunc32(ga);
+    if (maybe_above<R>(om32 * dtn32, 0.999f * ga32) && above(Om * P.dtn, ga)) {
       Om = ga * P.inv_dtn;
+      om32 = trunc32(Om);
       if (live) ++cnt.clamp;
     }
     // 5. omega_c (Eq. (1)) as hbar omega_c / m c^2; chi = eps_r Omega gamma,
     //    tested as 1.5 chi > 1.5 on the product epsc is formed from
     const R e1 = P.eps_r15 * Om * ga;
     const R epsc = e1 * ga;
-    if (live && above(e1, R(1.5))) ++cnt.chi;
+    if (live && maybe_above<R>(eps32 * om32 * ga32, 1.499f) && above(e1, R(1.5))) ++cnt.chi;
     // 6. Landau-Lifshitz loss (Eq. (4)): ledger and optional kick
     const R om2 = Om * Om;
     if (rr_mode >= PRAD_RR_LEDGER) ll.add(w * P.ll_coef * om2 * ua2);
@@ -1119,6 +1159,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
     }
     // 7. position x^{n+1}
     const R ign = rsq(R(1) + n2);
+    ig_last = ign;
     const R dtg = P.dtn * ign;
     R xn = x + dtg * nux, yn = y + dtg * nuy, zn = z;
     if (dims == 3) zn = z + dtg * nuz;
@@ -1157,7 +1198,8 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
           if (part && dN > R(1)) ++cnt.dn1;
         };
         if constexpr (sizeof(R) == 8) {
-          if (part && may_emit(P.tab32, w0, w1, w2, P.cn_dt * Om * dn_scale)) draw();
+          if (part && may_emit(P.tab32, w0, w1, w2, cn32 * om32 * static_cast<float>(dn_scale)))
+            draw();
         } else {
           draw();
         }

@@ -52,3 +52,29 @@ def test_fp64_records_equal_oracle(case, n_try, select):
     np.testing.assert_allclose(a[2], b[2], rtol=1e-6)
     np.testing.assert_allclose(a[3], b[3], rtol=1e-6)
     assert stats["dn_gt1"] == r["stats"]["dn_gt1"]
+
+
+@pytest.mark.parametrize("rr", [0, 1, 2])
+@pytest.mark.parametrize("e_field", [0.0, 1e9])
+def test_fp64_state_is_the_same_for_every_launch_shape(rr, e_field):
+    """Constant B, with and without E (whose zero terms a pure B field leaves
+    out), the LL ledger off, booked and applied: 1/gamma is carried from step
+    to step within a launch and formed anew at its start, to the same bits."""
+    wl = W.const_b(n=700, seed=3, rr_mode=rr)
+    wl.E = (0.0, e_field, 0.0)
+    got = []
+    for spl in (1, 7, 40):
+        ctx = prad.Context(wl.problem_kwargs(), precision=prad.PRAD_FP64, max_particles=wl.n,
+                           photon_capacity=1 << 14, steps_per_launch=spl)
+        st = ctx.to_device(wl.state)
+        ctx.push_emit(st, 40)
+        got.append({k: v.cpu().numpy() for k, v in st.items()})
+        ctx.close()
+    ref = wl.copy_state()
+    O.run(O.Problem(**wl.problem_kwargs()), ref, 40)
+    for k in ("x", "y", "z", "ux", "uy", "uz"):
+        np.testing.assert_array_equal(got[0][k], got[1][k], err_msg=k)
+        np.testing.assert_array_equal(got[0][k], got[2][k], err_msg=k)
+    u = np.stack([got[0][k] - ref[k] for k in ("ux", "uy", "uz")], 1)
+    n = np.linalg.norm(np.stack([ref[k] for k in ("ux", "uy", "uz")], 1), axis=1)
+    assert (np.linalg.norm(u, axis=1) <= 1e-12 * n).all()
