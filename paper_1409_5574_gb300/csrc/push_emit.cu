@@ -218,6 +218,13 @@ __device__ __forceinline__ float positive_part(float v) { return v > 0.0f ? v : 
 __device__ __forceinline__ double positive_part(double v) {
   return static_cast<uint32_t>(__double2hiint(v)) - 1u < 0x7ff00000u ? v : 0.0;
 }
+// x^2 + y^2 + z^2 with its roundings fixed (two places must give the same bits)
+__device__ __forceinline__ double norm2_rn(double x, double y, double z) {
+  return __fma_rn(z, z, __fma_rn(y, y, __dmul_rn(x, x)));
+}
+__device__ __forceinline__ float norm2_rn(float x, float y, float z) {
+  return x * x + y * y + z * z;
+}
 // A FP64 value >= 0 cut to FP32 by its bits (off by less than 2^-23 of it);
 // NaN outside FP32's normal range.  maybe_above: false only if such values
 // are not above each other; NaN says maybe.  FP32 steps compare directly.
@@ -1051,8 +1058,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
       // LL kick 1/gamma is the previous step's, from the same momentum)
       const R umx = ux, umy = uy, umz = uz;
       if (s == 0 || rr_mode == PRAD_RR_APPLY) {
-        const R m2 = umx * umx + umy * umy + umz * umz;
-        ig_last = rsq(R(1) + m2);
+        ig_last = rsq(R(1) + norm2_rn(umx, umy, umz));
       }
       const R igm = ig_last;
       const R tx = hq * f.Bx * igm, ty = hq * f.By * igm, tz = hq * f.Bz * igm;
@@ -1151,6 +1157,7 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
     const R om2 = Om * Om;
     if (rr_mode >= PRAD_RR_LEDGER) ll.add(w * P.ll_coef * om2 * ua2);
     R n2 = nux * nux + nuy * nuy + nuz * nuz;
+    if constexpr (sizeof(R) == 8) n2 = norm2_rn(nux, nuy, nuz);
     if (rr_mode == PRAD_RR_APPLY) {
       const R gL = sqr_pos(R(1) + n2);
       const R fk = rcp(R(1) + P.ll_coef * om2 * gL);
