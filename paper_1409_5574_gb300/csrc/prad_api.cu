@@ -699,6 +699,16 @@ bool ensure_bins(prad_ctx* c) {
   return true;
 }
 
+// Whether the context's stream is being captured (or cannot be asked).
+bool capturing(prad_ctx* c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
 // Whether a Yee launch takes the binned gather: FP32, table sampler, enough
 // particles and steps to pay for the binning, and no stream capture (whose
 // replays would share the scratch with other calls).
@@ -708,12 +718,7 @@ bool use_bins(prad_ctx* c, int64_t n, int32_t nsteps, int sub) {
       n * nsteps < (sub < kBinFused ? 2 : 1) * kBinMinWork ||
       c->cfg.max_particles >= (int64_t(1) << 31))
     return false;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return cs == cudaStreamCaptureStatusNone && ensure_bins(c);
+  return !capturing(c) && ensure_bins(c);
 }
 
 // Scratch for the sort: max_particles copies of the 7 state arrays and the
@@ -853,7 +858,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
         CK(c, launch_push_emit_tiled<float>(p, mw, 256, c->stream));
       }
       p.gate = b.work_count + 1;
-      CK(c, launch_push_emit<float>(p, f.kind, c->cfg.sampler, grid, block, c->stream));
+      CK(c, launch_push_emit<float>(p, f.kind, c->cfg.sampler, grid, block, c->stream, false));
       done += m;
     }
     CK(c, launch_tile_unbin(p, b, c->num_sms, c->stream));
@@ -968,6 +973,9 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
   if constexpr (sizeof(R) == 4) {
     if (binned) return push_binned(c, p, pp, nsteps, sub, grid, block);
   }
+  // launches overlap the drain of the one before (captured ones do not: the
+  // caller's graph keeps plain dependencies)
+  const bool pdl = !capturing(c);
   const uint64_t phase0 = p.phase_t0;
   for (int32_t done = 0; done < nsteps;) {
     const int32_t m = (nsteps - done) < sub ? (nsteps - done) : sub;
@@ -987,7 +995,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         continue;
       }
     }
-    CK(c, launch_push_emit<R>(p, c->fields.kind, c->cfg.sampler, grid, block, c->stream));
+    CK(c, launch_push_emit<R>(p, c->fields.kind, c->cfg.sampler, grid, block, c->stream, pdl));
     done += m;
   }
   return mlp_finish(c, c->d_led_emit);

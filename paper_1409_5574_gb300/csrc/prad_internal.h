@@ -243,7 +243,7 @@ int push_emit_occupancy(const StepParams<R>& p, int field_kind, int sampler, int
 int batch_max_blocks_per_sm(int block, int sampler, bool ctrl, bool std_cfg);
 template <typename R>
 cudaError_t launch_push_emit(const StepParams<R>& p, int field_kind, int sampler, int grid,
-                             int block, cudaStream_t s);
+                             int block, cudaStream_t s, bool pdl);
 template <typename R>
 cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
                                 R* x_out, R* g_out, int64_t n, cudaStream_t s);

@@ -1468,6 +1468,19 @@ __device__ __forceinline__ StepParams<R> spec_params(const StepParams<R>& in) {
 // PF: 0 no prefetch (multi-step launches); 1 one step per launch, the next
 // particle prefetched; 2 the same for a dense launch (see dense_launch).
 // PWS: the plane wave's signs at compile time (0: from the parameters).
+// A launch may start while the one before it on the stream drains (programmatic
+// stream serialisation): until pdl_wait it may read what no kernel writes (the
+// sampling table), then the earlier launches are complete and visible.  The
+// trigger follows the wait, so at most one launch waits behind a running one.
+// (1000 electrons, one step per launch: 5.3 us a launch without, 3.2 with; 2^24
+// one-step calls 4.07 against 3.98 ms per 16.)
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename R, int FIELD, int SAMP, int PF, int CTRL, bool STD = false, int PWS = 0>
 __global__ void __launch_bounds__(256, (PF ? PRAD_PF_MINB : MinBlocks<R, FIELD, SAMP>::value))
     k_push_emit(const StepParams<R> P_arg) {
@@ -1476,9 +1489,6 @@ __global__ void __launch_bounds__(256, (PF ? PRAD_PF_MINB : MinBlocks<R, FIELD, 
 #else
   const StepParams<R>& P = P_arg;
 #endif
-  if constexpr (FIELD == PRAD_FIELD_YEE2D) {  // behind a binned launch
-    if (P.gate && *P.gate == 0u) return;
-  }
   constexpr bool kSTab = kSharedTab<R, SAMP, PF, CTRL>;
   using Stage = typename std::conditional<
       CTRL == 2, PhotonStageSpread,
@@ -1489,6 +1499,11 @@ __global__ void __launch_bounds__(256, (PF ? PRAD_PF_MINB : MinBlocks<R, FIELD, 
   if constexpr (kSTab) {
     for (int k = threadIdx.x; k < kNTab; k += blockDim.x) stab[k] = __ldg(P.tab + k);
     __syncthreads();
+  }
+  pdl_wait();
+  pdl_trigger();
+  if constexpr (FIELD == PRAD_FIELD_YEE2D) {  // behind a binned launch
+    if (P.gate && *P.gate == 0u) return;
   }
   Stage& stage = stage_all[threadIdx.x >> 5];
   int fill = 0;  // warp-uniform
@@ -1787,26 +1802,42 @@ cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int blo
 }
 
 
+// pdl: the launch may begin before the stream's earlier work is done (pdl_wait).
+template <typename R>
+void launch_one(void (*kernel)(const StepParams<R>), const StepParams<R>& p, int grid, int block,
+                cudaStream_t s, bool pdl) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  (void)cudaLaunchKernelEx(&cfg, kernel, p);  // (the caller reads the last error)
+}
+
 template <typename R, int FIELD, int SAMP, int PF, int CTRL>
-void launch_k(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
+void launch_k(const StepParams<R>& p, int grid, int block, cudaStream_t s, bool pdl) {
   if constexpr (kHasStd<R, FIELD, CTRL>) {
     if (std_config(p, FIELD == PRAD_FIELD_YEE2D ? 2 : 3) && (CTRL != 2 || one_trial(p))) {
       // (the spread's kernel reads the signs: with them at compile time the
       // compiler contracts other products and the results change in the last bit)
       if constexpr (FIELD == PRAD_FIELD_PLANE_WAVE && CTRL != 2) {
         switch (pw_signs(p)) {
-          case 1: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 1><<<grid, block, 0, s>>>(p); return;
-          case 2: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 2><<<grid, block, 0, s>>>(p); return;
-          case 3: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 3><<<grid, block, 0, s>>>(p); return;
-          default: k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 4><<<grid, block, 0, s>>>(p); return;
+          case 1: launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 1>, p, grid, block, s, pdl); return;
+          case 2: launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 2>, p, grid, block, s, pdl); return;
+          case 3: launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 3>, p, grid, block, s, pdl); return;
+          default: launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, true, 4>, p, grid, block, s, pdl); return;
         }
       } else {
-        k_push_emit<R, FIELD, SAMP, PF, CTRL, true><<<grid, block, 0, s>>>(p);
+        launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, true>, p, grid, block, s, pdl);
         return;
       }
     }
   }
-  k_push_emit<R, FIELD, SAMP, PF, CTRL, false><<<grid, block, 0, s>>>(p);
+  launch_one(k_push_emit<R, FIELD, SAMP, PF, CTRL, false>, p, grid, block, s, pdl);
 }
 
 template <typename R, int FIELD, int SAMP, int PF, int CTRL>
@@ -1852,30 +1883,30 @@ bool stream_launch(const StepParams<R>&, int field_kind, int nsub) {
 
 template <typename R, int FIELD, int CTRL>
 cudaError_t launch_field_c(const StepParams<R>& p, int sampler, int grid, int block,
-                           cudaStream_t s) {
+                           cudaStream_t s, bool pdl) {
   if constexpr (CTRL == 2) {  // angular spread: table sampler, no prefetch variant
     if (sampler != PRAD_SAMPLER_TABLE) return cudaErrorInvalidValue;
-    launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, 2>(p, grid, block, s);
+    launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, 2>(p, grid, block, s, pdl);
     return cudaGetLastError();
   } else {
     if (sampler == PRAD_SAMPLER_TABLE) {
       if constexpr (kHasStream<R, FIELD>) {
         if (stream_launch(p, FIELD, p.nsub)) {
           if (dense_launch(p))
-            launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 2, CTRL>(p, grid, block, s);
+            launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 2, CTRL>(p, grid, block, s, pdl);
           else
-            launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 1, CTRL>(p, grid, block, s);
+            launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 1, CTRL>(p, grid, block, s, pdl);
           return cudaGetLastError();
         }
       }
-      launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, CTRL>(p, grid, block, s);
+      launch_k<R, FIELD, PRAD_SAMPLER_TABLE, 0, CTRL>(p, grid, block, s, pdl);
       return cudaGetLastError();
     }
     if constexpr (sizeof(R) == 4) {
       if (sampler == PRAD_SAMPLER_MLP)
-        launch_k<R, FIELD, PRAD_SAMPLER_MLP, 0, CTRL>(p, grid, block, s);
+        launch_k<R, FIELD, PRAD_SAMPLER_MLP, 0, CTRL>(p, grid, block, s, pdl);
       else
-        launch_k<R, FIELD, PRAD_SAMPLER_MLP_FALLBACK, 0, CTRL>(p, grid, block, s);
+        launch_k<R, FIELD, PRAD_SAMPLER_MLP_FALLBACK, 0, CTRL>(p, grid, block, s, pdl);
       return cudaGetLastError();
     }
     return cudaErrorInvalidValue;
@@ -1884,11 +1915,11 @@ cudaError_t launch_field_c(const StepParams<R>& p, int sampler, int grid, int bl
 
 template <typename R, int FIELD>
 cudaError_t launch_field(const StepParams<R>& p, int sampler, int grid, int block,
-                         cudaStream_t s) {
-  if (p.ang != nullptr) return launch_field_c<R, FIELD, 2>(p, sampler, grid, block, s);
+                         cudaStream_t s, bool pdl) {
+  if (p.ang != nullptr) return launch_field_c<R, FIELD, 2>(p, sampler, grid, block, s, pdl);
   const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
-  return ctrl ? launch_field_c<R, FIELD, 1>(p, sampler, grid, block, s)
-              : launch_field_c<R, FIELD, 0>(p, sampler, grid, block, s);
+  return ctrl ? launch_field_c<R, FIELD, 1>(p, sampler, grid, block, s, pdl)
+              : launch_field_c<R, FIELD, 0>(p, sampler, grid, block, s, pdl);
 }
 
 template <typename R, int FIELD, int CTRL>
@@ -1966,14 +1997,14 @@ template int push_emit_occupancy<double>(const StepParams<double>&, int, int, in
 
 template <typename R>
 cudaError_t launch_push_emit(const StepParams<R>& p, int field_kind, int sampler, int grid,
-                             int block, cudaStream_t s) {
+                             int block, cudaStream_t s, bool pdl) {
   switch (field_kind) {
     case PRAD_FIELD_CONST:
-      return launch_field<R, PRAD_FIELD_CONST>(p, sampler, grid, block, s);
+      return launch_field<R, PRAD_FIELD_CONST>(p, sampler, grid, block, s, pdl);
     case PRAD_FIELD_PLANE_WAVE:
-      return launch_field<R, PRAD_FIELD_PLANE_WAVE>(p, sampler, grid, block, s);
+      return launch_field<R, PRAD_FIELD_PLANE_WAVE>(p, sampler, grid, block, s, pdl);
     case PRAD_FIELD_YEE2D:
-      return launch_field<R, PRAD_FIELD_YEE2D>(p, sampler, grid, block, s);
+      return launch_field<R, PRAD_FIELD_YEE2D>(p, sampler, grid, block, s, pdl);
     default:
       return cudaErrorInvalidValue;
   }
@@ -2039,9 +2070,9 @@ cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
 }
 
 template cudaError_t launch_push_emit<float>(const StepParams<float>&, int, int, int, int,
-                                            cudaStream_t);
+                                            cudaStream_t, bool);
 template cudaError_t launch_push_emit<double>(const StepParams<double>&, int, int, int, int,
-                                             cudaStream_t);
+                                             cudaStream_t, bool);
 template cudaError_t launch_push_emit_tiled<float>(const StepParams<float>&, int, int, cudaStream_t);
 template cudaError_t launch_push_emit_tiled<double>(const StepParams<double>&, int, int, cudaStream_t);
 template cudaError_t launch_eval_sampler<float>(const StepParams<float>&, const uint32_t*, float*, float*, int64_t, cudaStream_t);
