@@ -58,7 +58,7 @@ struct prad_ctx {
   double* d_led_emit = nullptr;
   double* d_led_ll = nullptr;
   void* d_red = nullptr;
-  double* d_sums = nullptr;
+  double* d_sums = nullptr;      // after the counters, in their allocation
   // host-side totals folded in at each drain
   int64_t drained_records = 0;
   int64_t drained_dropped = 0;
@@ -1099,15 +1099,16 @@ int prad_init(prad_ctx** out, const prad_config* cfg) {
   // CTAs of at least 32 threads
   c->batch_busy_n = c->num_sms * 64;
   CKI(cudaMalloc(&c->d_batch_busy, sizeof(unsigned long long) * c->batch_busy_n));
-  CKI(cudaMalloc(&c->d_cnt, kNumCounters * sizeof(unsigned long long)));
+  // the counters, then the two sums of the energy budget: one read-back
+  CKI(cudaMalloc(&c->d_cnt, kNumCounters * sizeof(unsigned long long) + 2 * sizeof(double)));
   CKI(cudaMemset(c->d_cnt, 0, kNumCounters * sizeof(unsigned long long)));
+  c->d_sums = reinterpret_cast<double*>(c->d_cnt + kNumCounters);
   const size_t np = static_cast<size_t>(cfg->max_particles);
   CKI(cudaMalloc(&c->d_led_emit, np * sizeof(double)));
   CKI(cudaMalloc(&c->d_led_ll, np * sizeof(double)));
   CKI(cudaMemset(c->d_led_emit, 0, np * sizeof(double)));
   CKI(cudaMemset(c->d_led_ll, 0, np * sizeof(double)));
   CKI(cudaMalloc(&c->d_red, kLedgerScratchBytes));
-  CKI(cudaMalloc(&c->d_sums, 2 * sizeof(double)));
   // learned sampler: network, optimiser state, G^-1 table
   CKI(cudaMalloc(&c->d_mlp, sizeof(float) * kNumParams));
   CKI(cudaMalloc(&c->d_mlp_m, sizeof(float) * kNumParams));
@@ -1149,7 +1150,6 @@ int prad_destroy(prad_ctx* c) {
   cudaFree(c->d_led_emit);
   cudaFree(c->d_led_ll);
   cudaFree(c->d_red);
-  cudaFree(c->d_sums);
   cudaFree(c->d_mlp);
   cudaFree(c->d_mlp_m);
   cudaFree(c->d_mlp_v);
@@ -1292,11 +1292,11 @@ int prad_energy_budget(prad_ctx* c, double* emitted, double* rr_loss, prad_stats
   if (!c) return fail(c, PRAD_ERR_ARG, "energy_budget: null context");
   CK(c, launch_ledger_reduce(c->d_led_emit, c->d_led_ll, c->cfg.max_particles,
                              c->d_red, c->num_sms, c->d_sums, c->stream));
-  double sums[2];
-  unsigned long long cnt[kNumCounters];
-  CK(c, cudaMemcpyAsync(sums, c->d_sums, sizeof(sums), cudaMemcpyDeviceToHost, c->stream));
+  unsigned long long cnt[kNumCounters + 2];
   CK(c, cudaMemcpyAsync(cnt, c->d_cnt, sizeof(cnt), cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));
+  double sums[2];
+  std::memcpy(sums, cnt + kNumCounters, sizeof(sums));
   if (emitted) *emitted = sums[0];
   if (rr_loss) *rr_loss = sums[1];
   if (s) {
