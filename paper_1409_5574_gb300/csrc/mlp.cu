@@ -38,34 +38,36 @@ constexpr int kTB = 128;  // samples per block (one tile: one sample per thread)
 constexpr uint32_t kTrSbo64 = (kHid / 8) * 128;
 constexpr uint32_t kTrSbo128 = (kTB / 8) * 128;
 
-// Shared memory of the training kernel (~72 KB: three CTAs per SM).  The
-// operand tiles are in the canonical K-major layout of the tensor cores (no
-// swizzle, mlp_tc.cuh).  The forward operands are dead once the forward MMA
-// has completed, and the backward operands take their place; once the
-// backward MMAs have completed, dW2 (on its way to coalesced stores) takes
-// theirs and delta1 that of d2t and h1t.  The dW2 product reads its A operand
-// as 128 rows from d2t: rows 64..127 are h1t's bytes (d2t is followed by
-// h1t), and give TMEM lanes 64..127 that are never read.
-constexpr int kTW = kHid + 1;  // padded rows of dW2 (bank conflicts)
+// Shared memory of the training kernel (~56 KB: four CTAs per SM).  The
+// operand tiles are in the canonical layout of the tensor cores without
+// swizzle (mlp_tc.cuh), core matrices of 8 rows x 16 bytes.  The forward
+// operands are dead once the forward MMA has completed, and the backward
+// operands take their place; once the backward MMAs have completed, delta1
+// and dW2 (on its way to coalesced stores) take all of it.  delta2 [s][j] is
+// K-major for the dh1 product (K = j) and, read with the strides of its core
+// matrices exchanged, M-major for dW2 (M = j, K = s); that product's rows
+// 64..127 are whatever follows (the next samples' core matrices, W2^T at the
+// end), and give TMEM lanes 64..127 that are never read.
 struct alignas(128) TrainTcSmem {
   union {
     struct {
-      uint16_t a2[kTB * kTcK2];    // [h1 f16 | 1 1 0..] (forward layer 2, A)
-      uint16_t b2[kHid * kTcK2];   // halved W2 | split b2, f16 (forward layer 2, B)
-    } fwd;
-    struct {
-      uint16_t d2[kTB * kHid];     // bf16 delta2 [s][j] (delta1, A)
-      uint16_t w2t[kHid * kHid];   // BF16 W2^T [i][j] (delta1, B)
-    } bwd;
-    float dw2[kHid * kTW];         // dW2 [j][i]
-  } u;
-  union {
-    struct {
-      uint16_t d2t[kHid * kTB];    // bf16 delta2^T [j][s] (dW2, A rows 0..63)
-      uint16_t h1t[kHid * kTB];    // bf16(silu(z1))^T [i][s] (dW2, B)
+      union {
+        struct {
+          uint16_t a2[kTB * kTcK2];    // [h1 f16 | 1 1 0..] (forward layer 2, A)
+          uint16_t b2[kHid * kTcK2];   // halved W2 | split b2, f16 (forward layer 2, B)
+        } fwd;
+        struct {
+          uint16_t d2[kTB * kHid];     // bf16 delta2 [s][j] (A of dh1 and of dW2)
+          uint16_t w2t[kHid * kHid];   // BF16 W2^T [i][j] (dh1, B)
+        } bwd;
+      } u;
+      uint16_t h1t[kHid * kTB];        // bf16(silu(z1))^T [i][s] (dW2, B)
     } t;
-    float d1[kTB * kHid];          // delta1 [s][i], column i of row s at i ^ (s & 31)
-  } v;
+    struct {
+      float d1[kTB * kHid];            // delta1 [s][i], column i of row s at i ^ (s & 31)
+      float dw2[kHid * kHid];          // dW2 [j][i], the same exchange
+    } r;
+  } m;
   float wsum[kTB / 32][2 * kHid];  // per-warp sums of dL/dW3 and dL/db2
   float4 w1b1[kHid];               // (BF16 W1 row j, b1 j)
   float w3[kHid];
@@ -76,18 +78,20 @@ struct alignas(128) TrainTcSmem {
   uint32_t tmem;
   uint64_t bar;
 };
-static_assert(offsetof(TrainTcSmem, u.fwd.b2) % 128 == 0 &&
-                  offsetof(TrainTcSmem, u.bwd.w2t) % 128 == 0 &&
-                  offsetof(TrainTcSmem, v.t.d2t) % 128 == 0 &&
-                  offsetof(TrainTcSmem, v.t.h1t) ==
-                      offsetof(TrainTcSmem, v.t.d2t) + kHid * kTB * 2 &&
+static_assert(offsetof(TrainTcSmem, m.t.u.fwd.b2) % 128 == 0 &&
+                  offsetof(TrainTcSmem, m.t.u.bwd.w2t) % 128 == 0 &&
+                  offsetof(TrainTcSmem, m.t.h1t) % 128 == 0 &&
                   offsetof(TrainTcSmem, bar) % 8 == 0,
-              "operand and mbarrier alignment; h1t directly after d2t");
-static_assert(tc_off(kTB - 1, kTB - 1, kTrSbo128) < 2 * kHid * kTB &&
-                  tc_off(kHid - 1, kTB - 1, kTrSbo128) < kHid * kTB &&
+              "operand and mbarrier alignment");
+// strides of delta2's core matrices as dW2's A operand: along M (units j)
+// and along K (samples), and bytes per K = 16 step
+constexpr uint32_t kTrMSbo = 128, kTrMLbo = kTrSbo64, kTrMStep = 2 * kTrSbo64;
+static_assert(tc_off(kHid - 1, kTB - 1, kTrSbo128) < kHid * kTB &&
                   tc_off(kTB - 1, kHid - 1, kTrSbo64) < kTB * kHid &&
-                  tc_off(kHid - 1, kHid - 1, kTrSbo64) < kHid * kHid,
-              "training tiles stay inside their arrays (dW2's A: d2t and h1t)");
+                  tc_off(kHid - 1, kHid - 1, kTrSbo64) < kHid * kHid &&
+                  (kTB / 8 - 1) * kTrMLbo + (kTB / 8) * kTrMSbo <=
+                      sizeof(uint16_t) * (kTB * kHid + kHid * kHid),
+              "training tiles stay inside their arrays (dW2's A: d2 and w2t)");
 
 // Warp sums of 32 per-lane values v[0..31] (recursive halving: each round a
 // lane keeps one half of its range and adds its partner's copy of it); lane l
@@ -173,19 +177,36 @@ __device__ __forceinline__ bool train_wait(TrainTcSmem& S, uint32_t parity) {
 // A tensor-core wait that runs out zeroes the block's partials and sets
 // status bit 2.
 //
-// A block is short (one tile) and bound by latency, so what it loads is loaded
-// 16 bytes at a time and early, z1 is formed twice instead of kept (the block
-// then fits three times into an SM), and dW2 goes out in whole lines.  A batch
-// of 65536 samples: 76 us with element-wise images, a 33 KB z1 and two blocks
-// per SM, 36 us so (1.7 rounds of blocks are now 1.1).
-__global__ void __launch_bounds__(kTB, 3)
+// A block is short (one tile) and bound by latency and issue, so what it loads
+// is loaded 16 bytes at a time, z1 is formed twice instead of kept and delta2
+// kept once (four blocks then fit into an SM, and the 512 of a 65536-sample
+// batch run together), dW2 goes out in whole lines, and a launch draws its
+// samples while the reduction before it drains.  A batch of 65536 samples: 76
+// us with element-wise images, a 33 KB z1 and two blocks per SM, 36 us with
+// three, 29 us so.
+__global__ void __launch_bounds__(kTB, 4)
     k_mlp_train_tc(MlpDev dev, SampleSpec sp, float* __restrict__ partial,
                    float* __restrict__ loss_part, unsigned long long* status) {
   extern __shared__ unsigned char raw[];
   TrainTcSmem& S = *reinterpret_cast<TrainTcSmem*>(
       (reinterpret_cast<uintptr_t>(raw) + 127) & ~static_cast<uintptr_t>(127));
   const int s = threadIdx.x, lane = s & 31, warp = s >> 5;
-  // ---- set-up: weights on their way, then mbarrier, TMEM and the sample
+  // ---- set-up: mbarrier, TMEM and a drawn sample, which need nothing of the
+  // launch before; then the weights
+  if (s == 0) tc_mbar_init(&S.bar);
+  __syncwarp();
+  if (s < 32) tc_tmem_alloc(&S.tmem, 128);
+  const int64_t idx = static_cast<int64_t>(blockIdx.x) * kTB + s;
+  const bool valid = idx < sp.n_valid;
+  float f[4] = {0.0f, 0.0f, 0.0f, -1.0f}, tgt = 0.0f, wgt = 0.0f;
+  if (sp.explicit_samples) pdl_wait();  // (the caller's array)
+  if (valid) make_sample(sp, idx, f, &tgt, &wgt);  // (padding rows contribute nothing)
+  S.x[s][0] = f[0];
+  S.x[s][1] = f[1];
+  S.x[s][2] = f[2];
+  S.x[s][3] = f[3];
+  pdl_wait();
+  pdl_trigger();
   uint4 wq[4];  // W2 row n = e >> 3, units 8 (e & 7) .. + 7, e = s + 128 q
 #pragma unroll
   for (int q = 0; q < 4; ++q)
@@ -198,20 +219,7 @@ __global__ void __launch_bounds__(kTB, 3)
     w3v = dev.params[kOffW3 + s];
     b2v = dev.params[kOffB2 + s];
   }
-  if (s == 0) {
-    S.b3 = dev.params[kOffB3];
-    tc_mbar_init(&S.bar);
-  }
-  __syncwarp();
-  if (s < 32) tc_tmem_alloc(&S.tmem, 128);
-  const int64_t idx = static_cast<int64_t>(blockIdx.x) * kTB + s;
-  const bool valid = idx < sp.n_valid;
-  float f[4] = {0.0f, 0.0f, 0.0f, -1.0f}, tgt = 0.0f, wgt = 0.0f;
-  if (valid) make_sample(sp, idx, f, &tgt, &wgt);  // (padding rows contribute nothing)
-  S.x[s][0] = f[0];
-  S.x[s][1] = f[1];
-  S.x[s][2] = f[2];
-  S.x[s][3] = f[3];
+  if (s == 0) S.b3 = dev.params[kOffB3];
   // forward B (unit n, k): halved W2 | split b2
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(kTB, 3)
       out[h] = static_cast<uint32_t>(tc_f16_bits(a)) |
                (static_cast<uint32_t>(tc_f16_bits(b)) << 16);
     }
-    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(n, 8 * c, kTcSbo2)]) =
+    *reinterpret_cast<uint4*>(&S.m.t.u.fwd.b2[tc_off(n, 8 * c, kTcSbo2)]) =
         make_uint4(out[0], out[1], out[2], out[3]);
   }
   if (s < kHid) {
@@ -235,14 +243,14 @@ __global__ void __launch_bounds__(kTB, 3)
     const float hi = __half2float(__float2half_rn(hb));
     const uint32_t pk = static_cast<uint32_t>(tc_f16_bits(hi)) |
                         (static_cast<uint32_t>(tc_f16_bits(hb - hi)) << 16);
-    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(s, kHid, kTcSbo2)]) = make_uint4(pk, 0u, 0u, 0u);
-    *reinterpret_cast<uint4*>(&S.u.fwd.b2[tc_off(s, kHid + 8, kTcSbo2)]) =
+    *reinterpret_cast<uint4*>(&S.m.t.u.fwd.b2[tc_off(s, kHid, kTcSbo2)]) = make_uint4(pk, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(&S.m.t.u.fwd.b2[tc_off(s, kHid + 8, kTcSbo2)]) =
         make_uint4(0u, 0u, 0u, 0u);
   }
   // forward A columns 64..79: 1 1 0..
-  *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, kHid, kTcSbo2)]) =
+  *reinterpret_cast<uint4*>(&S.m.t.u.fwd.a2[tc_off(s, kHid, kTcSbo2)]) =
       make_uint4(0x3C003C00u, 0u, 0u, 0u);
-  *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, kHid + 8, kTcSbo2)]) =
+  *reinterpret_cast<uint4*>(&S.m.t.u.fwd.a2[tc_off(s, kHid + 8, kTcSbo2)]) =
       make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   // ---- layer 1 (FP32, BF16 weights)
@@ -258,14 +266,14 @@ __global__ void __launch_bounds__(kTB, 3)
     for (int q = 0; q < 8; ++q) {
       const int j = 8 * c + q;
       z[q] = z1(j);
-      S.v.t.h1t[tc_off(j, s, kTrSbo128)] = tc_bf16_bits(silu(z[q]));
+      S.m.t.h1t[tc_off(j, s, kTrSbo128)] = tc_bf16_bits(silu(z[q]));
     }
     uint4 q4;
     q4.x = silu_f16x2(z[0], z[1]);
     q4.y = silu_f16x2(z[2], z[3]);
     q4.z = silu_f16x2(z[4], z[5]);
     q4.w = silu_f16x2(z[6], z[7]);
-    *reinterpret_cast<uint4*>(&S.u.fwd.a2[tc_off(s, 8 * c, kTcSbo2)]) = q4;
+    *reinterpret_cast<uint4*>(&S.m.t.u.fwd.a2[tc_off(s, 8 * c, kTcSbo2)]) = q4;
   }
   tc_fence_proxy_async();
   tc_fence_before_sync();
@@ -275,8 +283,8 @@ __global__ void __launch_bounds__(kTB, 3)
   const uint32_t lanes = tmem + (static_cast<uint32_t>(s & ~31) << 16);
   // ---- forward layer 2 on the tensor cores
   if (s == 0) {
-    const uint64_t ad = tc_desc(S.u.fwd.a2, kTcLbo, kTcSbo2);
-    const uint64_t bd = tc_desc(S.u.fwd.b2, kTcLbo, kTcSbo2);
+    const uint64_t ad = tc_desc(S.m.t.u.fwd.a2, kTcLbo, kTcSbo2);
+    const uint64_t bd = tc_desc(S.m.t.u.fwd.b2, kTcLbo, kTcSbo2);
 #pragma unroll
     for (int k = 0; k < kTcK2 / 16; ++k)
       tc_mma_f16(tmem, ad + k * (kTcKStep >> 4), bd + k * (kTcKStep >> 4),
@@ -304,7 +312,7 @@ __global__ void __launch_bounds__(kTB, 3)
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int e = s + kTB * q, i = e & (kHid - 1), j = 8 * (e >> 6);
-      *reinterpret_cast<uint4*>(&S.u.bwd.w2t[tc_off(i, j, kTrSbo64)]) =
+      *reinterpret_cast<uint4*>(&S.m.t.u.bwd.w2t[tc_off(i, j, kTrSbo64)]) =
           make_uint4(wt[q][0], wt[q][1], wt[q][2], wt[q][3]);
     }
     // z2 = 2 c; output o = W3 h2 + b3 with h2 = f16(silu(z2)); loss, dL/do
@@ -340,12 +348,9 @@ __global__ void __launch_bounds__(kTB, 3)
         uint32_t pk[4];
 #pragma unroll
         for (int q = 0; q < 8; q += 2) {
-          const int j = 32 * half + 8 * c + q;
           pk[q / 2] = pack_bf16x2(v[8 * c + q], v[8 * c + q + 1]);
-          S.v.t.d2t[tc_off(j, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] & 0xffffu);
-          S.v.t.d2t[tc_off(j + 1, s, kTrSbo128)] = static_cast<uint16_t>(pk[q / 2] >> 16);
         }
-        *reinterpret_cast<uint4*>(&S.u.bwd.d2[tc_off(s, 32 * half + 8 * c, kTrSbo64)]) =
+        *reinterpret_cast<uint4*>(&S.m.t.u.bwd.d2[tc_off(s, 32 * half + 8 * c, kTrSbo64)]) =
             make_uint4(pk[0], pk[1], pk[2], pk[3]);
       }
       S.wsum[warp][kHid + 32 * half + lane] = warp_sum32(v, lane);
@@ -360,14 +365,14 @@ __global__ void __launch_bounds__(kTB, 3)
   __syncthreads();
   tc_fence_after_sync();
   if (!bad && s == 0) {
-    const uint64_t ad = tc_desc(S.v.t.d2t, kTcLbo, kTrSbo128),
-                   bd = tc_desc(S.v.t.h1t, kTcLbo, kTrSbo128);
+    const uint64_t ad = tc_desc(S.m.t.u.bwd.d2, kTrMLbo, kTrMSbo),
+                   bd = tc_desc(S.m.t.h1t, kTcLbo, kTrSbo128);
 #pragma unroll
     for (int k = 0; k < kTB / 16; ++k)
-      tc_mma_f16(tmem, ad + k * (kTcKStep >> 4), bd + k * (kTcKStep >> 4),
-                 tc_idesc(true, kTB, kHid), k > 0 ? 1u : 0u);
-    const uint64_t ad3 = tc_desc(S.u.bwd.d2, kTcLbo, kTrSbo64);
-    const uint64_t bd3 = tc_desc(S.u.bwd.w2t, kTcLbo, kTrSbo64);
+      tc_mma_f16(tmem, ad + k * (kTrMStep >> 4), bd + k * (kTcKStep >> 4),
+                 tc_idesc(true, kTB, kHid) | kTcMajorMA, k > 0 ? 1u : 0u);
+    const uint64_t ad3 = tc_desc(S.m.t.u.bwd.d2, kTcLbo, kTrSbo64);
+    const uint64_t bd3 = tc_desc(S.m.t.u.bwd.w2t, kTcLbo, kTrSbo64);
 #pragma unroll
     for (int k = 0; k < kHid / 16; ++k)
       tc_mma_f16(tmem + kHid, ad3 + k * (kTcKStep >> 4), bd3 + k * (kTcKStep >> 4),
@@ -387,7 +392,7 @@ __global__ void __launch_bounds__(kTB, 3)
         uint32_t v[32];
         tmem_ld_wait_32x32b_x32(lanes + 32 * half, v);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) S.u.dw2[s * kTW + 32 * half + q] = __uint_as_float(v[q]);
+        for (int q = 0; q < 32; ++q) S.m.r.dw2[s * kHid + ((32 * half + q) ^ lane)] = __uint_as_float(v[q]);
       }
     }
     // delta1 = dh1 silu'(z1)
@@ -398,7 +403,7 @@ __global__ void __launch_bounds__(kTB, 3)
 #pragma unroll
       for (int q = 0; q < 32; ++q) {
         const int i = 32 * half + q;
-        S.v.d1[s * kHid + (i ^ lane)] = __uint_as_float(v[q]) * silu_grad(z1(i));
+        S.m.r.d1[s * kHid + (i ^ lane)] = __uint_as_float(v[q]) * silu_grad(z1(i));
       }
     }
   }
@@ -414,7 +419,7 @@ __global__ void __launch_bounds__(kTB, 3)
   } else {
 #pragma unroll 8
     for (int e = s; e < kHid * kHid; e += kTB)
-      gp[kOffW2 + e] = S.u.dw2[(e / kHid) * kTW + (e & (kHid - 1))];
+      gp[kOffW2 + e] = S.m.r.dw2[(e & ~(kHid - 1)) + ((e & (kHid - 1)) ^ ((e / kHid) & 31))];
     // per-unit sums over the block's samples (FP32, sample 0 first): unit j,
     // two of its four sums per thread, beside one of the block's two
     const int j = s & (kHid - 1);
@@ -422,7 +427,7 @@ __global__ void __launch_bounds__(kTB, 3)
     if (s < kHid) {
 #pragma unroll 8
       for (int r = 0; r < kTB; ++r) {
-        const float d = S.v.d1[r * kHid + (j ^ (r & 31))];
+        const float d = S.m.r.d1[r * kHid + (j ^ (r & 31))];
         a = fmaf(d, S.x[r][0], a);
         b = fmaf(d, S.x[r][1], b);
         t += S.dout[r];
@@ -436,7 +441,7 @@ __global__ void __launch_bounds__(kTB, 3)
     } else {
 #pragma unroll 8
       for (int r = 0; r < kTB; ++r) {
-        const float d = S.v.d1[r * kHid + (j ^ (r & 31))];
+        const float d = S.m.r.d1[r * kHid + (j ^ (r & 31))];
         a = fmaf(d, S.x[r][2], a);
         b += d;
         t += S.loss[r];
@@ -472,6 +477,8 @@ __global__ void __launch_bounds__(kRedThreadsAdam)
                       __nv_bfloat16* __restrict__ w2, float lr, float b1t, float b2t, int apply,
                       float* __restrict__ loss_out, float loss_scale) {
   __shared__ float rows[kRedRows][kRedParams];
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int p = blockIdx.x * kRedParams + lane;
   // one address form for every lane (a branch around the load would keep the
@@ -650,6 +657,26 @@ __global__ void k_ginv_eval(const float* __restrict__ tab, const float* __restri
 
 }  // namespace
 
+namespace {
+// A launch that may begin while the one before it on the stream drains (its
+// kernel calls pdl_wait).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), int grid, int block, size_t dyn, cudaStream_t s,
+                       A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+}  // namespace
+
 size_t mlp_train_smem_bytes() { return sizeof(TrainTcSmem) + 128; }
 
 cudaError_t launch_mlp_train_block(const MlpDev& dev, uint32_t key0, uint32_t key1,
@@ -668,8 +695,7 @@ cudaError_t launch_mlp_train_block(const MlpDev& dev, uint32_t key0, uint32_t ke
   cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tc,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  k_mlp_train_tc<<<nblocks, kTB, bytes, s>>>(dev, sp, partial, loss_part, status);
-  return cudaGetLastError();
+  return launch_pdl(k_mlp_train_tc, nblocks, kTB, bytes, s, dev, sp, partial, loss_part, status);
 }
 
 cudaError_t launch_mlp_reduce_adam(const float* partial, int nblocks, const float* loss_part,
@@ -678,10 +704,8 @@ cudaError_t launch_mlp_reduce_adam(const float* partial, int nblocks, const floa
                                    int apply, float* loss_out, float loss_scale,
                                    cudaStream_t s) {
   const int blocks = (kNumParams + 1 + kRedParams - 1) / kRedParams;
-  k_mlp_reduce_adam<<<blocks, kRedThreadsAdam, 0, s>>>(partial, nblocks, loss_part, grad, params, m,
-                                                v, w2, lr, b1t, b2t, apply, loss_out,
-                                                loss_scale);
-  return cudaGetLastError();
+  return launch_pdl(k_mlp_reduce_adam, blocks, kRedThreadsAdam, 0, s, partial, nblocks, loss_part,
+                    grad, params, m, v, w2, lr, b1t, b2t, apply, loss_out, loss_scale);
 }
 
 // The tcgen05 kernels take more than 48 KB of dynamic shared memory: the

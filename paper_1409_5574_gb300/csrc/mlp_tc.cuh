@@ -152,6 +152,9 @@ __host__ __device__ constexpr uint32_t tc_idesc(bool bf16, int m, int n) {
          (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
 }
 
+// A is M-major (its core matrices hold 8 consecutive M of 8 K): bit 15.
+constexpr uint32_t kTcMajorMA = 1u << 15;
+
 // ---- 128-row tiles, one warpgroup per tile ----------------------------------
 constexpr int kTcRows = 128;          // rows per tile = threads per warpgroup
 // Warpgroups per CTA.  Each runs its own sequence of tiles (its A tile, its

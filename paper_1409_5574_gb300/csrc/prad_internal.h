@@ -65,6 +65,19 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __hiloint2double(static_cast<int>(hi), static_cast<int>(b << 29));
 }
 
+// A launch may start while the one before it on the stream drains (programmatic
+// stream serialisation): until pdl_wait it may read what no kernel writes (the
+// sampling table), then the earlier launches are complete and visible.  The
+// trigger follows the wait, so at most one launch waits behind a running one.
+// (1000 electrons, one step per launch: 5.3 us a launch without, 3.2 with; 2^24
+// one-step calls 4.07 against 3.98 ms per 16.)
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Counter slots of the per-context device counter array.
 enum Counter {
   kCursor = 0,   // photon append cursor (counts attempts, may exceed cap)

@@ -1468,19 +1468,6 @@ __device__ __forceinline__ StepParams<R> spec_params(const StepParams<R>& in) {
 // PF: 0 no prefetch (multi-step launches); 1 one step per launch, the next
 // particle prefetched; 2 the same for a dense launch (see dense_launch).
 // PWS: the plane wave's signs at compile time (0: from the parameters).
-// A launch may start while the one before it on the stream drains (programmatic
-// stream serialisation): until pdl_wait it may read what no kernel writes (the
-// sampling table), then the earlier launches are complete and visible.  The
-// trigger follows the wait, so at most one launch waits behind a running one.
-// (1000 electrons, one step per launch: 5.3 us a launch without, 3.2 with; 2^24
-// one-step calls 4.07 against 3.98 ms per 16.)
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-__device__ __forceinline__ void pdl_trigger() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 template <typename R, int FIELD, int SAMP, int PF, int CTRL, bool STD = false, int PWS = 0>
 __global__ void __launch_bounds__(256, (PF ? PRAD_PF_MINB : MinBlocks<R, FIELD, SAMP>::value))
     k_push_emit(const StepParams<R> P_arg) {
