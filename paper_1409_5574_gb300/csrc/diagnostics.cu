@@ -38,14 +38,17 @@ __device__ __noinline__ int exact_bin(const AngularArgs& a, float fx, float fy, 
 
 // The same from FP32 angles where these are sure of it.  The FP64 acos and
 // atan2 of every record kept the FP64 pipe (2 lanes per clock and SM) busy for
-// 1258 us on 6.3M records, 260 us so; only records closer to an edge than the
+// 1258 us on 6.3M records, 102 us so; only records closer to an edge than the
 // FP32 error take them now.  Bounds of that error: the three products and
 // sums of a component, of magnitude at most 1.0000002 with axes rounded to
 // FP32, are off by at most 3e-7 = kDot; so theta, and acosf adds at most
 // 4 ulp (1e-6): |dtheta| <= kDot / sin(theta) + 1e-6 while sin(theta) stays
-// above 1e-2 (beyond, the second-order term is below a hundredth of it), and
-// |dphi| <= 2 kDot / rho + 2e-6 with rho the length across the axis.  Directions
-// closer to the axis are left to FP64, and the margins are doubled.
+// above 1e-2 (the second-order term is then below a hundredth of it) and at
+// most sqrt(2 kDot) = 7.8e-4 closer to the axis, and |dphi| <= 2 kDot / rho +
+// 2e-6 with rho the length across the axis.  Directions within 1e-5 of the axis
+// are left to FP64, and the margins are doubled.  (The beam's own axis is where
+// a good part of the records lie: with every direction within 1e-2 of it left
+// to FP64 the kernel took 260 us.)
 struct FastBins {
   float ax[3], e1[3], e2[3], per_t, per_p;
   int ntheta, nphi;
@@ -68,12 +71,13 @@ struct FastBins {
     const float p2 = x * e2[0] + y * e2[1] + z * e2[2];
     const float rho2 = p1 * p1 + p2 * p2;
     // (a direction of another length than 1, or NaN, is left to FP64)
-    if (!(rho2 > 1e-4f && fabsf(rho2 + c * c - 1.0f) < 1e-5f)) return kUnsure;
+    if (!(rho2 > 1e-10f && fabsf(rho2 + c * c - 1.0f) < 1e-5f)) return kUnsure;
     const float inv = rsqrtf(rho2);
     const float t = acosf(c) * per_t;
     float ph = atan2f(p2, p1);
     ph = (ph < 0.0f ? ph + static_cast<float>(kTwoPi) : ph) * per_p;
-    const float mt = 2.0f * (kDot * inv + 1e-6f) * per_t + 2.4e-7f * t;
+    const float dt = rho2 > 1e-4f ? kDot * inv : 7.8e-4f;
+    const float mt = 2.0f * (dt + 1e-6f) * per_t + 2.4e-7f * t;
     const float mp = 2.0f * (2.0f * kDot * inv + 2e-6f) * per_p + 2.4e-7f * ph;
     if (fabsf(t - rintf(t)) <= mt || fabsf(ph - rintf(ph)) <= mp) return kUnsure;
     const int it = static_cast<int>(t), ip = static_cast<int>(ph);
@@ -82,7 +86,12 @@ struct FastBins {
   }
 };
 
-__global__ void k_angular_hist(AngularArgs a) {
+// 512 threads share a block's bins, two blocks per SM: the adds are compare and
+// swap loops on shared memory, whose latency wants warps to hide it, while
+// every block more adds its bins to the output once more (256 x 2: 152 us, 512
+// x 2: 102, 512 x 3: 128, 1024 x 1: 108 on 6.3M records).
+constexpr int kHistThreads = 512, kHistBlocks = 2;
+__global__ void __launch_bounds__(kHistThreads, kHistBlocks) k_angular_hist(AngularArgs a) {
   extern __shared__ double hist[];
   const int nb = a.ntheta * a.nphi;
   for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0.0;
@@ -108,7 +117,7 @@ __global__ void k_angular_hist(AngularArgs a) {
 
 }  // namespace
 
-cudaError_t launch_angular_hist(const AngularArgs& a, int grid, cudaStream_t s) {
+cudaError_t launch_angular_hist(const AngularArgs& a, int num_sms, cudaStream_t s) {
   const size_t smem = sizeof(double) * static_cast<size_t>(a.ntheta) * a.nphi;
   cudaError_t e = cudaFuncSetAttribute(k_angular_hist,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -116,7 +125,7 @@ cudaError_t launch_angular_hist(const AngularArgs& a, int grid, cudaStream_t s) 
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(a.out, 0, smem, s);
   if (e != cudaSuccess) return e;
-  k_angular_hist<<<grid, 256, smem, s>>>(a);
+  k_angular_hist<<<kHistBlocks * num_sms, kHistThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 

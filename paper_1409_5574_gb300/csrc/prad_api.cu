@@ -1281,7 +1281,7 @@ int prad_angular_histogram(prad_ctx* c, const double axis[3], const double ref[3
   a.cap = c->cfg.photon_capacity;
   if (!c->d_hist) CK(c, cudaMalloc(&c->d_hist, sizeof(double) * kMaxAngularBins));
   a.out = c->d_hist;
-  CK(c, launch_angular_hist(a, c->num_sms * 2, c->stream));
+  CK(c, launch_angular_hist(a, c->num_sms, c->stream));
   const size_t nb = static_cast<size_t>(ntheta) * nphi;
   CK(c, cudaMemcpyAsync(out, c->d_hist, sizeof(double) * nb, cudaMemcpyDeviceToHost, c->stream));
   CK(c, cudaStreamSynchronize(c->stream));

@@ -325,7 +325,7 @@ struct AngularArgs {
   int32_t ntheta, nphi;
   double* out;                   // device, ntheta x nphi
 };
-cudaError_t launch_angular_hist(const AngularArgs& a, int grid, cudaStream_t s);
+cudaError_t launch_angular_hist(const AngularArgs& a, int num_sms, cudaStream_t s);
 int mlp_finish_blocks_per_sm();
 cudaError_t launch_ginv_eval(const float* tab, const float* r, float* out, int64_t n,
                              cudaStream_t s);
