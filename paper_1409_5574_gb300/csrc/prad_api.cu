@@ -852,7 +852,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
       const int rc = spec_for(c, p, true, &spec);
       if (rc != PRAD_OK) return rc;
       if (spec) {
-        CK(c, spec_launch(spec, p, mw, 256, c->stream));
+        CK(c, spec_launch(spec, p, mw, 256, c->stream, false));
         ++c->spec_launches;
       } else {
         CK(c, launch_push_emit_tiled<float>(p, mw, 256, c->stream));
@@ -920,7 +920,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         p.work_count = c->bins.work_count;
         const int mw = static_cast<int>(max_work_items(n, ntx * nty, chunk));
         if (spec) {
-          CK(c, spec_launch(spec, p, mw, 256, c->stream));
+          CK(c, spec_launch(spec, p, mw, 256, c->stream, false));
           ++c->spec_launches;
         } else {
           CK(c, launch_push_emit_tiled<R>(p, mw, 256, c->stream));
@@ -989,7 +989,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         if (rc != PRAD_OK) return rc;
       }
       if (spec) {
-        CK(c, spec_launch(spec, p, grid, block, c->stream));
+        CK(c, spec_launch(spec, p, grid, block, c->stream, pdl));
         ++c->spec_launches;
         done += m;
         continue;

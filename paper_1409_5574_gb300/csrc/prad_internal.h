@@ -357,9 +357,10 @@ cudaError_t spec_get(SpecCache* c, int device, const StepParams<float>& p, const
                      const SpecFn** out, char* msg, size_t msg_len);
 int spec_occupancy(const SpecFn* f, int block);
 // grid blocks of block threads; the tiled kernel gets its tile's dynamic
-// shared memory
+// shared memory.  pdl: as launch_push_emit's (not for the tiled kernel, which
+// does not wait for the launch before itself)
 cudaError_t spec_launch(const SpecFn* f, const StepParams<float>& p, int grid, int block,
-                        cudaStream_t s);
+                        cudaStream_t s, bool pdl);
 // Whether a launch with these parameters runs a specialisable variant (FP32
 // standard configuration of the plane wave or the Yee grid, no control or
 // diagnostics; the tiled kernel with the table sampler), and which.

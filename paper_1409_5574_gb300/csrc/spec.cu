@@ -66,7 +66,7 @@ struct Driver {
   decltype(&cuModuleLoadData) load = nullptr;
   decltype(&cuModuleUnload) unload = nullptr;
   decltype(&cuModuleGetFunction) get_function = nullptr;
-  decltype(&cuLaunchKernel) launch = nullptr;
+  decltype(&cuLaunchKernelEx) launch = nullptr;
   decltype(&cuOccupancyMaxActiveBlocksPerMultiprocessor) occupancy = nullptr;
   decltype(&cuCtxGetCurrent) ctx_current = nullptr;
   decltype(&cuFuncSetAttribute) set_attr = nullptr;
@@ -127,7 +127,7 @@ const Driver& driver() {
   static std::once_flag once;
   std::call_once(once, [] {
     d.ok = entry("cuModuleLoadData", &d.load) && entry("cuModuleUnload", &d.unload) &&
-           entry("cuModuleGetFunction", &d.get_function) && entry("cuLaunchKernel", &d.launch) &&
+           entry("cuModuleGetFunction", &d.get_function) && entry("cuLaunchKernelEx", &d.launch) &&
            entry("cuOccupancyMaxActiveBlocksPerMultiprocessor", &d.occupancy) &&
            entry("cuCtxGetCurrent", &d.ctx_current) &&
            entry("cuFuncSetAttribute", &d.set_attr);
@@ -372,7 +372,7 @@ int spec_occupancy(const SpecFn* f, int block) {
 }
 
 cudaError_t spec_launch(const SpecFn* f, const StepParams<float>& p, int grid, int block,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool pdl) {
   const Driver& d = driver();
   CUcontext cur = nullptr;
   int prev = -1;
@@ -385,8 +385,19 @@ cudaError_t spec_launch(const SpecFn* f, const StepParams<float>& p, int grid, i
     if (d.ctx_current(&cur) != CUDA_SUCCESS || cur != f->ctx) return cudaErrorInvalidResourceHandle;
   }
   void* args[] = {const_cast<StepParams<float>*>(&p)};
-  const CUresult r = d.launch(f->fn, static_cast<unsigned>(grid), 1, 1, static_cast<unsigned>(block),
-                              1, 1, f->dyn_smem, reinterpret_cast<CUstream>(s), args, nullptr);
+  CUlaunchConfig cfg{};
+  cfg.gridDimX = static_cast<unsigned>(grid);
+  cfg.gridDimY = cfg.gridDimZ = 1;
+  cfg.blockDimX = static_cast<unsigned>(block);
+  cfg.blockDimY = cfg.blockDimZ = 1;
+  cfg.sharedMemBytes = f->dyn_smem;
+  cfg.hStream = reinterpret_cast<CUstream>(s);
+  CUlaunchAttribute at[1];
+  at[0].id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
+  at[0].value.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  const CUresult r = d.launch(&cfg, f->fn, args, nullptr);
   if (prev >= 0 && prev != f->device) cudaSetDevice(prev);
   switch (r) {
     case CUDA_SUCCESS: return cudaSuccess;
