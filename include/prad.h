@@ -97,8 +97,8 @@ typedef struct prad_config {
                                steps and gather from shared-memory field
                                tiles (0 = particles stay in the caller's
                                order: long FP32 calls gather through tiles
-                               from a reordered copy, 44 B x max_particles
-                               of context scratch, short ones from the
+                               from a reordered copy, 44 B per particle of
+                               context scratch, short ones from the
                                planes)                                    */
   int32_t batch_chunk;      /* push_emit_batch: particles per work item
                                (0 = 2048); multiple of 32                 */

@@ -652,7 +652,11 @@ int64_t max_work_items(int64_t n, int ntiles, int chunk) {
   return n / chunk + (n < ntiles ? n : ntiles) + 1;
 }
 
-// Particles per work item of a tiled launch of m steps.
+// Particles per work item of a tiled launch of m steps: an eighth of what
+// would give every resident block (three per SM) one item, so that the last
+// round of blocks is a small part of the launch, but enough particle-steps to
+// pay for a tile's staging.  (2^22 electrons in items of 4096, 1025 for 456
+// blocks, took 4003 us per 50 steps, in items of 1280 3816.)
 int chunk_of(int64_t n, int32_t m, int num_sms) {
   const int64_t even = n / (8 * 3 * static_cast<int64_t>(num_sms));
   const int64_t least = 16384 / (m > 0 ? m : 1);
@@ -673,15 +677,18 @@ void free_bins(BinBuffers& b) {
   b = BinBuffers{};
 }
 
-// Scratch of the binned gather; false (and nothing held) if it cannot be had.
-bool ensure_bins(prad_ctx* c) {
+// Scratch of the binned gather for n particles (44 bytes each); false (and
+// nothing held) if it cannot be had.
+bool ensure_bins(prad_ctx* c, int64_t n) {
   int ntx, nty;
-  const int ntiles = tile_counts(c->fields, &ntx, &nty);
+  int ntiles = tile_counts(c->fields, &ntx, &nty);
   BinBuffers& b = c->bins;
-  if (b.capacity >= c->cfg.max_particles && b.ntiles >= ntiles) return true;
+  if (b.capacity >= n && b.ntiles >= ntiles) return true;
+  if (n < b.capacity) n = b.capacity;
+  if (ntiles < b.ntiles) ntiles = b.ntiles;
   free_bins(b);
-  const size_t np = static_cast<size_t>(c->cfg.max_particles);
-  const int64_t mw = max_work_items(c->cfg.max_particles, ntiles, kChunkMin);
+  const size_t np = static_cast<size_t>(n);
+  const int64_t mw = max_work_items(n, ntiles, kChunkMin);
   if (cudaMalloc(&b.keys, np * sizeof(uint2)) != cudaSuccess ||
       cudaMalloc(&b.slot, np * sizeof(uint32_t)) != cudaSuccess ||
       cudaMalloc(&b.aos, np * 2 * sizeof(float4)) != cudaSuccess ||
@@ -694,7 +701,7 @@ bool ensure_bins(prad_ctx* c) {
     free_bins(b);
     return false;
   }
-  b.capacity = c->cfg.max_particles;
+  b.capacity = n;
   b.ntiles = ntiles;
   return true;
 }
@@ -718,7 +725,7 @@ bool use_bins(prad_ctx* c, int64_t n, int32_t nsteps, int sub) {
       n * nsteps < (sub < kBinFused ? 2 : 1) * kBinMinWork ||
       c->cfg.max_particles >= (int64_t(1) << 31))
     return false;
-  return !capturing(c) && ensure_bins(c);
+  return !capturing(c);
 }
 
 // Scratch for the sort: max_particles copies of the 7 state arrays and the
@@ -764,7 +771,9 @@ int sort_fp64(prad_ctx* c, const prad_particles* pp, int64_t n, int chunk = kChu
 
 // The FP32 state of p into the tile order of c->bins (the caller holds bin_mu).
 int bin_fp32(prad_ctx* c, const StepParams<float>& p, int chunk) {
-  if (!ensure_bins(c)) return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
+  // (once for all sizes, so that later calls can be captured)
+  if (!ensure_bins(c, c->cfg.max_particles))
+    return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
   const prad_fields& f = c->fields;
   int ntx, nty;
   BinBuffers b = c->bins;
@@ -959,6 +968,10 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
   if constexpr (sizeof(R) == 4) {
     p.nsub = sub_eff;
     binned = use_bins(c, n, nsteps, sub);
+    if (binned) {
+      std::lock_guard<std::mutex> lk(c->bin_mu);
+      binned = ensure_bins(c, n);
+    }
     const int rc = binned ? PRAD_OK : spec_for(c, p, false, &spec);
     if (rc != PRAD_OK) return rc;
   }
