@@ -1031,9 +1031,14 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
   // Two steps per iteration on the analytic fields in FP32 (the end of one
   // overlaps the start of the next; 2^22 electrons, 100 steps: 4123 against
   // 4007 us, with run-time specialised constants 3607 against 3567 on a late
-  // stretch).  Three or more outgrow the registers, and the Yee step is too
-  // long for two (2^22 sorted electrons 8331 against 8370 us).
-  constexpr int kUnroll = sizeof(R) == 4 && FIELD != PRAD_FIELD_YEE2D ? 2 : 1;
+  // stretch).  Three or more outgrow the registers; the Yee step is too long
+  // for two (2^22 sorted electrons 8331 against 8370 us), and so is the
+  // batched kernel's, whose parameters take registers (64 ensembles 3690
+  // against 3712 us; it and the control kernels stage by field).
+  constexpr int kUnroll = sizeof(R) == 4 && FIELD != PRAD_FIELD_YEE2D &&
+                                  !std::is_same<ST, PhotonStageSoA>::value
+                              ? 2
+                              : 1;
 #pragma unroll kUnroll
   for (int s = 0; s < nsub; ++s) {
     const uint32_t step = static_cast<uint32_t>(P.t0 + s);
