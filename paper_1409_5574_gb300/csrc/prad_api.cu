@@ -629,17 +629,20 @@ void free_sort(SortBuffers& b) {
 }
 
 // The binned gather: a call takes it from kBinMinSteps steps and kBinMinWork
-// particle-steps on (launches of fewer than kBinFused steps: twice that), and
-// bins its particles again every kBinSteps steps (they drift off the staged
-// halo).  Measured, plain against binned, 4 steps and 8 steps in one launch:
-// 2^20 particles in random order 649 against 289 and 1290 against 359 us, in
-// cell order (whose plain gather hits L1) 188 against 249 and 426 against
-// 325 us; 2^17 particles, 8 steps: 194 against 146 and 79 against 135 us.
-// 8 one-step launches: 2^20 random 1467 against 656, in cell order 513
-// against 610; 2^23 11440 against 3973 and 3574 against 3299 us.
+// particle-steps on, and bins its particles again every kBinSteps steps (they
+// drift off the staged halo).  Measured, plain against binned, 4 steps and 8
+// steps in one launch: 2^20 particles in random order 649 against 289 and 1290
+// against 329 us, in cell order (whose plain gather hits L1) 188 against 249 and
+// 423 against 327 us; 2^17 particles, 8 steps: 194 against 146 and 79 against
+// 135 us.  Launches of fewer than kBinFused steps stage a tile for few
+// particle-steps each: they take it from four times that work on, if the grid
+// holds kBinPerTile particles per tile (8 one-step launches, 2^20 in cell order
+// 514 against 607 us, 16 of them 1207 against 1133; 40 of 2^18 spread over a 4096^2
+// grid 2134 against 2448).
 constexpr int32_t kBinMinSteps = 8;
 constexpr int64_t kBinMinWork = int64_t(1) << 22;
 constexpr int kBinFused = 4;
+constexpr int64_t kBinPerTile = 64;
 constexpr int32_t kBinSteps = 50;
 
 int tile_counts(const prad_fields& f, int* ntx, int* nty) {
@@ -722,9 +725,11 @@ bool capturing(prad_ctx* c) {
 bool use_bins(prad_ctx* c, int64_t n, int32_t nsteps, int sub) {
   if (c->fields.kind != PRAD_FIELD_YEE2D || c->cfg.precision != PRAD_FP32 ||
       c->cfg.sampler != PRAD_SAMPLER_TABLE || nsteps < kBinMinSteps ||
-      n * nsteps < (sub < kBinFused ? 2 : 1) * kBinMinWork ||
+      n * nsteps < (sub < kBinFused ? 4 : 1) * kBinMinWork ||
       c->cfg.max_particles >= (int64_t(1) << 31))
     return false;
+  int ntx, nty;
+  if (sub < kBinFused && n < kBinPerTile * tile_counts(c->fields, &ntx, &nty)) return false;
   return !capturing(c);
 }
 

@@ -38,7 +38,7 @@ def _problem(nx, ny, n, seed, spread):
 
 def _run(wl, calls, per_launch, pid, **kw):
     off = 3
-    ctx = prad.Context(wl.problem_kwargs(), photon_capacity=1 << 21, max_particles=wl.n + off,
+    ctx = prad.Context(wl.problem_kwargs(), photon_capacity=1 << 23, max_particles=wl.n + off,
                        steps_per_launch=per_launch, **kw)
     st = ctx.to_device(wl.state)
     if pid:  # ids in another order than the particles'
@@ -62,7 +62,7 @@ def _run(wl, calls, per_launch, pid, **kw):
 
 @pytest.mark.parametrize("nx,ny,n,spread,steps,per_launch,pid,kw", [
     (130, 100, 524301, True, 8, 8, False, {}),         # tiles cut by the grid's end
-    (130, 100, 153001, True, 55, 1, True, {}),         # binned twice, one step per launch
+    (130, 100, 306001, True, 55, 1, True, {}),         # binned twice, one step per launch
     (40, 300, 480007, True, 9, 4, False, {}),          # narrower than the staged region
     (37, 29, 70001, False, 60, 60, False, {}),         # one launch longer than the interval
     (4129, 4100, 524301, True, 8, 8, True, {}),        # sparse: the plain kernel stands in
@@ -72,12 +72,12 @@ def _run(wl, calls, per_launch, pid, **kw):
 ])
 def test_binned_equals_plain(nx, ny, n, spread, steps, per_launch, pid, kw):
     wl = _problem(nx, ny, n, seed=nx + n, spread=spread)
-    assert n * steps >= (1 << 22) and (per_launch >= 4 or n * steps >= (1 << 23))
+    assert n * steps >= (1 << 22) and (per_launch >= 4 or n * steps >= (1 << 24))
     a = _run(wl, [1] * steps, 1, pid, **dict(kw, specialize=False))
     b = _run(wl, [steps], per_launch, pid, **kw)
     for k in a[0]:
         np.testing.assert_array_equal(a[0][k], b[0][k], err_msg=k)
-    assert 100 < len(a[1]) < 1 << 21
+    assert 100 < len(a[1]) < 1 << 23
     np.testing.assert_array_equal(a[1], b[1])
     np.testing.assert_allclose(a[2], b[2], rtol=1e-13, atol=0)
     np.testing.assert_allclose(a[3], b[3], rtol=1e-13, atol=0)
