@@ -73,13 +73,16 @@ struct FastBins {
     // (a direction of another length than 1, or NaN, is left to FP64)
     if (!(rho2 > 1e-10f && fabsf(rho2 + c * c - 1.0f) < 1e-5f)) return kUnsure;
     const float inv = rsqrtf(rho2);
-    const float t = acosf(c) * per_t;
+    // (c rounds beyond +-1 close to the axis or its opposite, and acosf is NaN
+    // there: clamped as the definition does, which moves c no further off)
+    const float t = acosf(fminf(fmaxf(c, -1.0f), 1.0f)) * per_t;
     float ph = atan2f(p2, p1);
     ph = (ph < 0.0f ? ph + static_cast<float>(kTwoPi) : ph) * per_p;
     const float dt = rho2 > 1e-4f ? kDot * inv : 7.8e-4f;
     const float mt = 2.0f * (dt + 1e-6f) * per_t + 2.4e-7f * t;
     const float mp = 2.0f * (2.0f * kDot * inv + 2e-6f) * per_p + 2.4e-7f * ph;
-    if (fabsf(t - rintf(t)) <= mt || fabsf(ph - rintf(ph)) <= mp) return kUnsure;
+    // (written so that a NaN is unsure)
+    if (!(fabsf(t - rintf(t)) > mt && fabsf(ph - rintf(ph)) > mp)) return kUnsure;
     const int it = static_cast<int>(t), ip = static_cast<int>(ph);
     if (it >= ntheta) return -1;
     return ip < nphi ? it * nphi + ip : kUnsure;
