@@ -699,7 +699,7 @@ bool ensure_bins(prad_ctx* c, int64_t n) {
       cudaMalloc(&b.starts, sizeof(unsigned int) * (ntiles + 1)) != cudaSuccess ||
       cudaMalloc(&b.cursor, sizeof(unsigned int) * ntiles) != cudaSuccess ||
       cudaMalloc(&b.work, sizeof(int4) * mw) != cudaSuccess ||
-      cudaMalloc(&b.work_count, 2 * sizeof(unsigned int)) != cudaSuccess) {
+      cudaMalloc(&b.work_count, kWorkWords * sizeof(unsigned int)) != cudaSuccess) {
     cudaGetLastError();  // the plain gather needs none of it
     free_bins(b);
     return false;
@@ -749,7 +749,7 @@ int ensure_sort(prad_ctx* c, size_t elem) {
   CK(c, cudaMalloc(&b.cursor, sizeof(unsigned int) * ntiles));
   const int64_t mw = max_work_items(c->cfg.max_particles, ntiles, kChunkMin);
   CK(c, cudaMalloc(&b.work, sizeof(int4) * mw));
-  CK(c, cudaMalloc(&b.work_count, sizeof(unsigned int)));
+  CK(c, cudaMalloc(&b.work_count, kWorkWords * sizeof(unsigned int)));
   b.capacity = c->cfg.max_particles;
   b.ntiles = ntiles;
   b.max_work = static_cast<int32_t>(mw);

@@ -184,6 +184,9 @@ constexpr int kStageW = kTile + 2 * kHalo;
 constexpr int kTileSmemBytes = 6 * kStageW * kStageW * 4;
 constexpr int kChunk = 4096;     // particles per work item of the tiled kernel at most
 constexpr int kChunkMin = 512;   // and at least (sizes the work list)
+// words of work_count, all written by the scan: work items, and the gate of the
+// plain kernel (0 where the scan is not asked for one)
+constexpr int kWorkWords = 2;
 
 struct SortBuffers {
   void* tmp[7];               // scratch copies of x y z ux uy uz w
