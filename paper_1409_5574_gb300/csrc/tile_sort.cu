@@ -15,15 +15,26 @@ namespace prad {
 
 namespace {
 
+// (v - v0) inv reduced to [0, n), with every rounding fixed.  Several kernels
+// find a particle's cell and must agree to the bit: a block reserves its run
+// of a tile from one count and fills it from another, so two contractions of
+// these products and sums would write beyond the run.
+__device__ __forceinline__ float wrapped(float v, float v0, float inv, float n) {
+  const float c = __fmul_rn(__fsub_rn(v, v0), inv);
+  return __fmaf_rn(-n, floor(__fdiv_rn(c, n)), c);
+}
+__device__ __forceinline__ double wrapped(double v, double v0, double inv, double n) {
+  const double c = __dmul_rn(__dsub_rn(v, v0), inv);
+  return __fma_rn(-n, floor(__ddiv_rn(c, n)), c);
+}
+
 // The grid cell (ix, iy) that holds (x, y): periodic, clamped (also for NaN)
 // into range.
 template <typename R>
 __device__ __forceinline__ int2 cell_xy(R x, R y, int nx, int ny, R x0, R y0, R inv_dx,
                                         R inv_dy) {
-  R xi = (x - x0) * inv_dx, yi = (y - y0) * inv_dy;
   const R fx = static_cast<R>(nx), fy = static_cast<R>(ny);
-  xi -= fx * floor(xi / fx);
-  yi -= fy * floor(yi / fy);
+  const R xi = wrapped(x, x0, inv_dx, fx), yi = wrapped(y, y0, inv_dy, fy);
   int ix = static_cast<int>(fmin(fmax(xi, R(0)), fx - R(1)));
   int iy = static_cast<int>(fmin(fmax(yi, R(0)), fy - R(1)));
   ix = ix < 0 ? 0 : (ix >= nx ? nx - 1 : ix);
