@@ -645,10 +645,13 @@ constexpr int kBinFused = 4;
 constexpr int64_t kBinPerTile = 64;
 constexpr int32_t kBinSteps = 50;
 
-int tile_counts(const prad_fields& f, int* ntx, int* nty) {
-  *ntx = (f.nx + kTile - 1) / kTile;
-  *nty = (f.ny + kTile - 1) / kTile;
+int tile_counts(int nx, int ny, int* ntx, int* nty) {
+  *ntx = (nx + kTile - 1) / kTile;
+  *nty = (ny + kTile - 1) / kTile;
   return (*ntx) * (*nty);
+}
+int tile_counts(const prad_fields& f, int* ntx, int* nty) {
+  return tile_counts(f.nx, f.ny, ntx, nty);
 }
 
 int64_t max_work_items(int64_t n, int ntiles, int chunk) {
@@ -680,11 +683,11 @@ void free_bins(BinBuffers& b) {
   b = BinBuffers{};
 }
 
-// Scratch of the binned gather for n particles (44 bytes each); false (and
-// nothing held) if it cannot be had.
-bool ensure_bins(prad_ctx* c, int64_t n) {
-  int ntx, nty;
-  int ntiles = tile_counts(c->fields, &ntx, &nty);
+// Scratch of the binned gather for n particles (44 bytes each) on ntiles
+// tiles; false (and nothing held) if it cannot be had.  The caller holds
+// bin_mu, up to the last launch that reads the scratch: another thread's call
+// may replace it.
+bool ensure_bins(prad_ctx* c, int64_t n, int ntiles) {
   BinBuffers& b = c->bins;
   if (b.capacity >= n && b.ntiles >= ntiles) return true;
   if (n < b.capacity) n = b.capacity;
@@ -776,15 +779,14 @@ int sort_fp64(prad_ctx* c, const prad_particles* pp, int64_t n, int chunk = kChu
 
 // The FP32 state of p into the tile order of c->bins (the caller holds bin_mu).
 int bin_fp32(prad_ctx* c, const StepParams<float>& p, int chunk) {
-  // (once for all sizes, so that later calls can be captured)
-  if (!ensure_bins(c, c->cfg.max_particles))
-    return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
-  const prad_fields& f = c->fields;
   int ntx, nty;
+  const int ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
+  // (once for all sizes, so that later calls can be captured)
+  if (!ensure_bins(c, c->cfg.max_particles, ntiles))
+    return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
   BinBuffers b = c->bins;
-  b.ntiles = tile_counts(f, &ntx, &nty);
-  CK(c, launch_tile_bin(p, b, f.x0, f.y0, 1.0 / f.dx, 1.0 / f.dy, chunk, false, c->num_sms,
-                        c->stream));
+  b.ntiles = ntiles;
+  CK(c, launch_tile_bin(p, b, chunk, false, c->num_sms, c->stream));
   return PRAD_OK;
 }
 
@@ -839,14 +841,18 @@ int spec_for(prad_ctx* c, const StepParams<float>& p, bool tiled, const SpecFn**
 // between run the tile-staged kernel on the copy, and it is written back.
 // Where the particles turn out to be sparse nothing is copied, the tile work
 // is empty and the plain kernel (grid, block) behind each launch runs instead
-// (a word on the device decides, nothing is read back).
+// (a word on the device decides, nothing is read back).  *taken: false if the
+// scratch cannot be had, and nothing was launched.
 int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int32_t nsteps,
-                int sub, int grid, int block) {
+                int sub, int grid, int block, bool* taken) {
+  // (one lock for the scratch and everything that is launched on it)
   std::lock_guard<std::mutex> lk(c->bin_mu);
-  const prad_fields& f = c->fields;
   int ntx, nty;
+  const int ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
+  *taken = ensure_bins(c, p.n, ntiles);
+  if (!*taken) return PRAD_OK;
   BinBuffers b = c->bins;
-  b.ntiles = tile_counts(f, &ntx, &nty);
+  b.ntiles = ntiles;
   p.ntx = ntx;
   p.aos = b.aos;
   p.work = b.work;
@@ -854,8 +860,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   const int chunk = chunk_of(p.n, sub < nsteps ? sub : nsteps, c->num_sms);
   const int mw = static_cast<int>(max_work_items(p.n, b.ntiles, chunk));
   for (int32_t done = 0; done < nsteps;) {
-    CK(c, launch_tile_bin(p, b, f.x0, f.y0, 1.0 / f.dx, 1.0 / f.dy, chunk, true, c->num_sms,
-                          c->stream));
+    CK(c, launch_tile_bin(p, b, chunk, true, c->num_sms, c->stream));
     const int32_t end = done + kBinSteps;
     while (done < nsteps && done < end) {
       const int32_t m = (nsteps - done) < sub ? (nsteps - done) : sub;
@@ -872,7 +877,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
         CK(c, launch_push_emit_tiled<float>(p, mw, 256, c->stream));
       }
       p.gate = b.work_count + 1;
-      CK(c, launch_push_emit<float>(p, f.kind, c->cfg.sampler, grid, block, c->stream, false));
+      CK(c, launch_push_emit<float>(p, p.field_kind, c->cfg.sampler, grid, block, c->stream, false));
       done += m;
     }
     CK(c, launch_tile_unbin(p, b, c->num_sms, c->stream));
@@ -913,7 +918,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
     if (n > c->cfg.max_particles)
       return fail(c, PRAD_ERR_ARG, "push_emit: n exceeds max_particles (sort scratch)");
     int ntx, nty;
-    tile_counts(c->fields, &ntx, &nty);
+    tile_counts(p.nx, p.ny, &ntx, &nty);
     p.ntx = ntx;
     const int interval = c->cfg.sort_interval;
     for (int32_t done = 0; done < nsteps;) {
@@ -969,28 +974,27 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
   // persistent grid: at most the resident blocks of the kernel variant, so
   // no block waits for a second wave (blocks_per_sm = 0: all of them)
   const SpecFn* spec = nullptr;
-  bool binned = false;
+  auto grid_of = [&] {
+    const int occ = spec ? spec_occupancy(spec, block)
+                         : push_emit_occupancy<R>(p, c->fields.kind, c->cfg.sampler, sub_eff,
+                                                  block, ctrl_of(c));
+    const int bps =
+        c->cfg.blocks_per_sm > 0 && c->cfg.blocks_per_sm < occ ? c->cfg.blocks_per_sm : occ;
+    const int64_t want = (n + block - 1) / block;
+    const int64_t cap = static_cast<int64_t>(c->num_sms) * bps;
+    return static_cast<int>(want < cap ? want : cap);
+  };
   if constexpr (sizeof(R) == 4) {
     p.nsub = sub_eff;
-    binned = use_bins(c, n, nsteps, sub);
-    if (binned) {
-      std::lock_guard<std::mutex> lk(c->bin_mu);
-      binned = ensure_bins(c, n);
+    if (use_bins(c, n, nsteps, sub)) {
+      bool taken = false;
+      const int rc = push_binned(c, p, pp, nsteps, sub, grid_of(), block, &taken);
+      if (rc != PRAD_OK || taken) return rc;
     }
-    const int rc = binned ? PRAD_OK : spec_for(c, p, false, &spec);
+    const int rc = spec_for(c, p, false, &spec);
     if (rc != PRAD_OK) return rc;
   }
-  const int occ = spec ? spec_occupancy(spec, block)
-                       : push_emit_occupancy<R>(p, c->fields.kind, c->cfg.sampler, sub_eff,
-                                                block, ctrl_of(c));
-  const int bps = c->cfg.blocks_per_sm > 0 && c->cfg.blocks_per_sm < occ ? c->cfg.blocks_per_sm
-                                                                         : occ;
-  const int64_t want = (n + block - 1) / block;
-  const int64_t cap = static_cast<int64_t>(c->num_sms) * bps;
-  const int grid = static_cast<int>(want < cap ? want : cap);
-  if constexpr (sizeof(R) == 4) {
-    if (binned) return push_binned(c, p, pp, nsteps, sub, grid, block);
-  }
+  const int grid = grid_of();
   // launches overlap the drain of the one before (captured ones do not: the
   // caller's graph keeps plain dependencies)
   const bool pdl = !capturing(c);

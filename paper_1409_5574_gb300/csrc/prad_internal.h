@@ -277,9 +277,8 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
 // tile); gate: sparse particles leave that to the plain kernel.
 // launch_tile_unbin writes the state back to where it came from,
 // launch_tile_unsort in its new order, with the weights and ids.
-cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
-                            double inv_dx, double inv_dy, int chunk, bool gate, int num_sms,
-                            cudaStream_t s);
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool gate,
+                            int num_sms, cudaStream_t s);
 cudaError_t launch_tile_unsort(const StepParams<float>& p, const BinBuffers& b, float* w,
                                uint32_t* pid, int num_sms, cudaStream_t s);
 cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, int num_sms,

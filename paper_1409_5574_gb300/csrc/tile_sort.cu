@@ -472,9 +472,8 @@ int stream_grid(int64_t n, int num_sms) {
 
 }  // namespace
 
-cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, double x0, double y0,
-                            double inv_dx, double inv_dy, int chunk, bool gate, int num_sms,
-                            cudaStream_t s) {
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool gate,
+                            int num_sms, cudaStream_t s) {
   const int64_t n = p.n;
   const float *x = p.x, *y = p.y;
   BinGeom g;
@@ -482,10 +481,10 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, dou
   g.ny = p.ny;
   g.ntx = (p.nx + kTile - 1) / kTile;
   g.ntiles = b.ntiles;
-  g.x0 = static_cast<float>(x0);
-  g.y0 = static_cast<float>(y0);
-  g.inv_dx = static_cast<float>(inv_dx);
-  g.inv_dy = static_cast<float>(inv_dy);
+  g.x0 = p.x0;
+  g.y0 = p.y0;
+  g.inv_dx = p.inv_dx;
+  g.inv_dy = p.inv_dy;
   cudaError_t e = cudaMemsetAsync(b.counts, 0, sizeof(unsigned int) * b.ntiles, s);
   if (e != cudaSuccess) return e;
   const bool sm = b.ntiles <= kBinTiles;
