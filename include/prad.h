@@ -98,8 +98,8 @@ typedef struct prad_config {
                                tiles (0 = particles stay in the caller's
                                order: long FP32 calls gather through tiles
                                from a reordered copy, 44 B per particle of
-                               context scratch, short ones from the
-                               planes)                                    */
+                               context scratch (prad_reserve_binning), short
+                               ones from the planes)                      */
   int32_t batch_chunk;      /* push_emit_batch: particles per work item
                                (0 = 2048); multiple of 32                 */
   int32_t use_graph;        /* push_emit_batch: capture the launches of a
@@ -349,6 +349,19 @@ int prad_autotune_batch(prad_ctx* ctx, const prad_ensemble* ens, int32_t n_ens,
  * (max_particles x 44 B, FP64 60 B).  Errors: PRAD_ERR_STATE (fields not YEE2D),
  * PRAD_ERR_ARG (null arrays, no pid array, n > max_particles). */
 int prad_sort_by_tile(prad_ctx* ctx, const prad_particles* p, int64_t n);
+
+/* Scratch of long unsorted FP32 Yee calls (prad_config.sort_interval = 0):
+ * they take 44 B per particle (and 28 B per tile) at the first such call and
+ * keep it for the context; more particles than it holds double it.
+ * on = 1 takes the scratch for max_particles and the current grid now, so
+ * that no later prad_push_emit allocates unless a prad_set_fields brings
+ * more tiles.  on = 0 frees it (waits for the stream; kept if prad_sort_by_tile
+ * has used it) and lets those calls gather from the planes, as short ones do,
+ * until a call with on = 1.  The results are the same.  (A measure of the
+ * implementation; the paper has no such quantity.)
+ * Errors: PRAD_ERR_STATE (on = 1 and the fields are not YEE2D), PRAD_ERR_CUDA
+ * (no memory: calls then gather from the planes). */
+int prad_reserve_binning(prad_ctx* ctx, int32_t on);
 
 /* Load balance of the last prad_push_emit_batch call (a measurement of the
  * batched form; the paper defines no such quantity): each CTA of its

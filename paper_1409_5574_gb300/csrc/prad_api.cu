@@ -68,6 +68,8 @@ struct prad_ctx {
   // a time, since a binning and the launches that read it belong together
   BinBuffers bins{};
   std::mutex bin_mu;
+  bool bins_off = false;         // prad_reserve_binning(ctx, 0)
+  bool bins_sorted = false;      // a sort has used the scratch (its captures may hold it)
   // learned sampler
   float* d_mlp = nullptr;        // FP32 master parameters
   float* d_mlp_m = nullptr;      // Adam moments
@@ -671,6 +673,14 @@ int chunk_of(int64_t n, int32_t m, int num_sms) {
   return static_cast<int>(c < kChunkMin ? kChunkMin : (c > kChunk ? kChunk : c));
 }
 
+// The calling thread may allocate and free while other threads capture their
+// streams (the capture stays valid).
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 void free_bins(BinBuffers& b) {
   cudaFree(b.keys);
   cudaFree(b.slot);
@@ -684,13 +694,17 @@ void free_bins(BinBuffers& b) {
 }
 
 // Scratch of the binned gather for n particles (44 bytes each) on ntiles
-// tiles; false (and nothing held) if it cannot be had.  The caller holds
-// bin_mu, up to the last launch that reads the scratch: another thread's call
-// may replace it.
+// tiles; false (and nothing held) if it cannot be had.  Particles beyond the
+// scratch double it (up to max_particles), so that a set that grows from call
+// to call is not allocated again each time.  The caller holds bin_mu, up to
+// the last launch that reads the scratch: another thread's call may replace it.
 bool ensure_bins(prad_ctx* c, int64_t n, int ntiles) {
   BinBuffers& b = c->bins;
   if (b.capacity >= n && b.ntiles >= ntiles) return true;
-  if (n < b.capacity) n = b.capacity;
+  if (n > b.capacity)
+    n = std::max(n, std::min(b.capacity ? 2 * b.capacity : n + n / 8, c->cfg.max_particles));
+  else
+    n = b.capacity;
   if (ntiles < b.ntiles) ntiles = b.ntiles;
   free_bins(b);
   const size_t np = static_cast<size_t>(n);
@@ -722,14 +736,18 @@ bool capturing(prad_ctx* c) {
   return cs != cudaStreamCaptureStatusNone;
 }
 
+// Whether the context's Yee calls may take the binned gather.
+bool can_bin(const prad_ctx* c) {
+  return c->cfg.precision == PRAD_FP32 && c->cfg.sampler == PRAD_SAMPLER_TABLE &&
+         c->cfg.max_particles < (int64_t(1) << 31);
+}
+
 // Whether a Yee launch takes the binned gather: FP32, table sampler, enough
 // particles and steps to pay for the binning, and no stream capture (whose
 // replays would share the scratch with other calls).
 bool use_bins(prad_ctx* c, int64_t n, int32_t nsteps, int sub) {
-  if (c->fields.kind != PRAD_FIELD_YEE2D || c->cfg.precision != PRAD_FP32 ||
-      c->cfg.sampler != PRAD_SAMPLER_TABLE || nsteps < kBinMinSteps ||
-      n * nsteps < (sub < kBinFused ? 4 : 1) * kBinMinWork ||
-      c->cfg.max_particles >= (int64_t(1) << 31))
+  if (c->fields.kind != PRAD_FIELD_YEE2D || !can_bin(c) || nsteps < kBinMinSteps ||
+      n * nsteps < (sub < kBinFused ? 4 : 1) * kBinMinWork)
     return false;
   int ntx, nty;
   if (sub < kBinFused && n < kBinPerTile * tile_counts(c->fields, &ntx, &nty)) return false;
@@ -784,6 +802,7 @@ int bin_fp32(prad_ctx* c, const StepParams<float>& p, int chunk) {
   // (once for all sizes, so that later calls can be captured)
   if (!ensure_bins(c, c->cfg.max_particles, ntiles))
     return fail(c, PRAD_ERR_CUDA, "tile sort: no device memory for its scratch");
+  c->bins_sorted = true;
   BinBuffers b = c->bins;
   b.ntiles = ntiles;
   CK(c, launch_tile_bin(p, b, chunk, false, c->num_sms, c->stream));
@@ -849,7 +868,10 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   std::lock_guard<std::mutex> lk(c->bin_mu);
   int ntx, nty;
   const int ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
-  *taken = ensure_bins(c, p.n, ntiles);
+  {
+    RelaxedCapture relaxed;
+    *taken = !c->bins_off && ensure_bins(c, p.n, ntiles);
+  }
   if (!*taken) return PRAD_OK;
   BinBuffers b = c->bins;
   b.ntiles = ntiles;
@@ -1237,6 +1259,26 @@ int prad_sort_by_tile(prad_ctx* c, const prad_particles* p, int64_t n) {
   if (n == 0) return PRAD_OK;
   if (c->cfg.precision == PRAD_FP32) return sort_fp32(c, p, n);
   return sort_fp64(c, p, n);
+}
+
+int prad_reserve_binning(prad_ctx* c, int32_t on) {
+  if (!c) return fail(c, PRAD_ERR_ARG, "reserve_binning: null context");
+  std::lock_guard<std::mutex> lk(c->bin_mu);
+  c->bins_off = on == 0;
+  RelaxedCapture relaxed;
+  if (!on) {
+    if (c->bins_sorted || !c->bins.capacity) return PRAD_OK;
+    CK(c, cudaStreamSynchronize(c->stream));
+    free_bins(c->bins);
+    return PRAD_OK;
+  }
+  if (!c->fields_set || c->fields.kind != PRAD_FIELD_YEE2D)
+    return fail(c, PRAD_ERR_STATE, "reserve_binning: fields are not YEE2D");
+  if (!can_bin(c)) return PRAD_OK;
+  int ntx, nty;
+  if (!ensure_bins(c, c->cfg.max_particles, tile_counts(c->fields, &ntx, &nty)))
+    return fail(c, PRAD_ERR_CUDA, "reserve_binning: no device memory for the scratch");
+  return PRAD_OK;
 }
 
 int prad_get_photons(prad_ctx* c, prad_photons* out, int64_t cap, int64_t* n_out,

@@ -90,6 +90,7 @@ SIGNATURES = {
     "prad_set_fields": (_i32, [_vp, ctypes.POINTER(prad_fields)]),
     "prad_push_emit": (_i32, [_vp, ctypes.POINTER(prad_particles), _i64, _i32]),
     "prad_sort_by_tile": (_i32, [_vp, ctypes.POINTER(prad_particles), _i64]),
+    "prad_reserve_binning": (_i32, [_vp, _i32]),
     "prad_push_emit_batch": (_i32, [_vp, ctypes.POINTER(prad_ensemble), _i32, _i32]),
     "prad_autotune_batch": (_i32, [_vp, ctypes.POINTER(prad_ensemble), _i32, _i32, _i64,
                                    ctypes.POINTER(prad_tuning)]),
@@ -174,6 +175,10 @@ def prad_push_emit(h, p: prad_particles, n: int, nsteps: int) -> int:
 
 def prad_sort_by_tile(h, p: prad_particles, n: int) -> int:
     return _check(load_library().prad_sort_by_tile(h, ctypes.byref(p), n), h)
+
+
+def prad_reserve_binning(h, on: bool) -> None:
+    _check(load_library().prad_reserve_binning(h, int(on)), h)
 
 
 def prad_push_emit_batch(h, ens, nsteps: int) -> int:
@@ -481,6 +486,12 @@ class Context:
     def sort_by_tile(self, st: Dict, pid0: int = 0, ledger_offset: int = 0) -> None:
         n = st["x"].numel()
         prad_sort_by_tile(self.h, self._particles(st, 0, pid0, ledger_offset), n)
+
+    def reserve_binning(self, on: bool = True) -> None:
+        """Take the scratch of long unsorted Yee calls now (``push_emit`` then
+        allocates nothing), or with ``on=False`` give it back and let those
+        calls gather from the planes."""
+        prad_reserve_binning(self.h, on)
 
     def photons(self, drain: bool = False, on_device: bool = True,
                 cap: Optional[int] = None) -> Dict:
