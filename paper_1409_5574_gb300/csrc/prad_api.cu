@@ -638,14 +638,20 @@ void free_sort(SortBuffers& b) {
 // 423 against 327 us; 2^17 particles, 8 steps: 194 against 146 and 79 against
 // 135 us.  Launches of fewer than kBinFused steps stage a tile for few
 // particle-steps each: they take it from four times that work on, if the grid
-// holds kBinPerTile particles per tile (8 one-step launches, 2^20 in cell order
+// holds kBinSparse particles per tile (8 one-step launches, 2^20 in cell order
 // 514 against 607 us, 16 of them 1207 against 1133; 40 of 2^18 spread over a 4096^2
 // grid 2134 against 2448).
+// Counting, scanning and the work list take 1 to 2 ns per tile of the grid, and
+// a sparse set pays for it in vain: a binning is tried only where kBinTileWork
+// particle-steps per tile follow, at 0.1 ns each (clumps) to 0.9 (2^19
+// electrons, 8 steps: over a 4096^2 grid 1390 us tried in vain against 1330
+// plain, within 256^2 cells of it 250 against 564; on 16384^2, where it is not
+// tried, 3560, tried in vain 4390; there 50 steps within 256^2 cells 1010 against 3430).
 constexpr int32_t kBinMinSteps = 8;
 constexpr int64_t kBinMinWork = int64_t(1) << 22;
 constexpr int kBinFused = 4;
-constexpr int64_t kBinPerTile = 64;
 constexpr int32_t kBinSteps = 50;
+constexpr int64_t kBinTileWork = 64;
 
 int tile_counts(int nx, int ny, int* ntx, int* nty) {
   *ntx = (nx + kTile - 1) / kTile;
@@ -744,14 +750,28 @@ bool can_bin(const prad_ctx* c) {
 
 // Whether a Yee launch takes the binned gather: FP32, table sampler, enough
 // particles and steps to pay for the binning, and no stream capture (whose
-// replays would share the scratch with other calls).
-bool use_bins(prad_ctx* c, int64_t n, int32_t nsteps, int sub) {
-  if (c->fields.kind != PRAD_FIELD_YEE2D || !can_bin(c) || nsteps < kBinMinSteps ||
+// replays would share the scratch with other calls).  *gate: the particles may
+// turn out to be too sparse, so that the plain kernel stands behind each
+// launch.
+bool use_bins(prad_ctx* c, const StepParams<float>& p, int32_t nsteps, int sub, bool* gate) {
+  const int64_t n = p.n;
+  if (p.field_kind != PRAD_FIELD_YEE2D || !can_bin(c) || nsteps < kBinMinSteps ||
       n * nsteps < (sub < kBinFused ? 4 : 1) * kBinMinWork)
     return false;
   int ntx, nty;
-  if (sub < kBinFused && n < kBinPerTile * tile_counts(c->fields, &ntx, &nty)) return false;
+  const int64_t ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
+  *gate = n < kBinSparse * ntiles;
+  if (*gate && sub < kBinFused) return false;
+  if (n * std::min(nsteps, kBinSteps) < kBinTileWork * ntiles) return false;
   return !capturing(c);
+}
+
+// Blocks of a tiled launch of at most mw work items: eight for every resident
+// one (three per SM), each taking more than one item only where there are
+// more.  (A block per possible item, most of them empty where the particles
+// fill a part of the grid, costs about 0.9 ns each.)
+int tiled_grid(int64_t mw, int num_sms) {
+  return static_cast<int>(std::min<int64_t>(mw, 8 * 3 * static_cast<int64_t>(num_sms)));
 }
 
 // Scratch for the sort: max_particles copies of the 7 state arrays and the
@@ -858,12 +878,14 @@ int spec_for(prad_ctx* c, const StepParams<float>& p, bool tiled, const SpecFn**
 // A Yee push of particles that stay in the caller's order: every kBinSteps
 // steps the state is copied in the order of tiles and cells, the launches in
 // between run the tile-staged kernel on the copy, and it is written back.
-// Where the particles turn out to be sparse nothing is copied, the tile work
-// is empty and the plain kernel (grid, block) behind each launch runs instead
-// (a word on the device decides, nothing is read back).  *taken: false if the
-// scratch cannot be had, and nothing was launched.
+// gate: where the particles turn out to be sparse nothing is copied, the tile
+// work is empty and the plain kernel (grid, block) behind each launch runs
+// instead (a word on the device decides, nothing is read back).  A specialised
+// context compiles one kernel for a call: the tiled one (1.06 times the
+// compiled-in one's speed), or with a gate the plain one (plain).
+// *taken: false if the scratch cannot be had, and nothing was launched.
 int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int32_t nsteps,
-                int sub, int grid, int block, bool* taken) {
+                int sub, bool gate, const SpecFn* plain, int grid, int block, bool* taken) {
   // (one lock for the scratch and everything that is launched on it)
   std::lock_guard<std::mutex> lk(c->bin_mu);
   int ntx, nty;
@@ -879,27 +901,33 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   p.aos = b.aos;
   p.work = b.work;
   p.work_count = b.work_count;
+  const SpecFn* spec = nullptr;  // (of every launch, whatever its steps)
+  const int rc = gate ? PRAD_OK : spec_for(c, p, true, &spec);
+  if (rc != PRAD_OK) return rc;
   const int chunk = chunk_of(p.n, sub < nsteps ? sub : nsteps, c->num_sms);
-  const int mw = static_cast<int>(max_work_items(p.n, b.ntiles, chunk));
+  const int tgrid = tiled_grid(max_work_items(p.n, ntiles, chunk), c->num_sms);
   for (int32_t done = 0; done < nsteps;) {
-    CK(c, launch_tile_bin(p, b, chunk, true, c->num_sms, c->stream));
+    CK(c, launch_tile_bin(p, b, chunk, gate, c->num_sms, c->stream));
     const int32_t end = done + kBinSteps;
     while (done < nsteps && done < end) {
       const int32_t m = (nsteps - done) < sub ? (nsteps - done) : sub;
       p.t0 = pp->t0 + done;
       p.nsub = m;
       p.gate = nullptr;
-      const SpecFn* spec = nullptr;
-      const int rc = spec_for(c, p, true, &spec);
-      if (rc != PRAD_OK) return rc;
       if (spec) {
-        CK(c, spec_launch(spec, p, mw, 256, c->stream, false));
+        CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
         ++c->spec_launches;
       } else {
-        CK(c, launch_push_emit_tiled<float>(p, mw, 256, c->stream));
+        CK(c, launch_push_emit_tiled<float>(p, tgrid, 256, c->stream));
       }
       p.gate = b.work_count + 1;
-      CK(c, launch_push_emit<float>(p, p.field_kind, c->cfg.sampler, grid, block, c->stream, false));
+      if (gate && plain) {
+        CK(c, spec_launch(plain, p, grid, block, c->stream, false));
+        ++c->spec_launches;
+      } else if (gate) {
+        CK(c, launch_push_emit<float>(p, p.field_kind, c->cfg.sampler, grid, block, c->stream,
+                                      false));
+      }
       done += m;
     }
     CK(c, launch_tile_unbin(p, b, c->num_sms, c->stream));
@@ -959,12 +987,12 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         p.aos = c->bins.aos;
         p.work = c->bins.work;
         p.work_count = c->bins.work_count;
-        const int mw = static_cast<int>(max_work_items(n, ntx * nty, chunk));
+        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms);
         if (spec) {
-          CK(c, spec_launch(spec, p, mw, 256, c->stream, false));
+          CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
           ++c->spec_launches;
         } else {
-          CK(c, launch_push_emit_tiled<R>(p, mw, 256, c->stream));
+          CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream));
         }
         CK(c, launch_tile_unsort(p, c->bins, static_cast<float*>(pp->w), pp->pid, c->num_sms,
                                  c->stream));
@@ -973,8 +1001,8 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         if (rc != PRAD_OK) return rc;
         p.work = c->sort.work;
         p.work_count = c->sort.work_count;
-        const int64_t mw = max_work_items(n, c->sort.ntiles, chunk);
-        CK(c, launch_push_emit_tiled<R>(p, static_cast<int>(mw), 256, c->stream));
+        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms);
+        CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream));
       }
       done += m;
     }
@@ -1008,9 +1036,12 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
   };
   if constexpr (sizeof(R) == 4) {
     p.nsub = sub_eff;
-    if (use_bins(c, n, nsteps, sub)) {
+    bool gate = false;
+    if (use_bins(c, p, nsteps, sub, &gate)) {
       bool taken = false;
-      const int rc = push_binned(c, p, pp, nsteps, sub, grid_of(), block, &taken);
+      int rc = gate ? spec_for(c, p, false, &spec) : PRAD_OK;
+      if (rc == PRAD_OK)
+        rc = push_binned(c, p, pp, nsteps, sub, gate, spec, gate ? grid_of() : 0, block, &taken);
       if (rc != PRAD_OK || taken) return rc;
     }
     const int rc = spec_for(c, p, false, &spec);

@@ -187,6 +187,9 @@ constexpr int kChunkMin = 512;   // and at least (sizes the work list)
 // words of work_count, all written by the scan: work items, and the gate of the
 // plain kernel (0 where the scan is not asked for one)
 constexpr int kWorkWords = 2;
+// Binned gather: below this many particles per occupied tile the plain kernel
+// gathers from global memory (a tile's staging would not pay).
+constexpr int kBinSparse = 64;
 
 struct SortBuffers {
   void* tmp[7];               // scratch copies of x y z ux uy uz w
@@ -266,7 +269,7 @@ cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
                           uint32_t* out, int64_t n, cudaStream_t s);
 template <typename R>
-cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int block,
+cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block,
                                    cudaStream_t s);
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,

@@ -1695,53 +1695,58 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   const StepParams<R>& P = P_arg;
 #endif
   constexpr bool kAos = sizeof(R) == 4;
-  if (blockIdx.x >= *P.work_count) return;
+  const unsigned int items = *P.work_count;
+  if (blockIdx.x >= items) return;
   extern __shared__ __align__(16) float tile_sm[];
   using Stage = typename std::conditional<CTRL == 2, PhotonStageSpread, PhotonStageSoA>::type;
   __shared__ Stage stage_all[kMaxWarps];
-  const int4 wk = P.work[blockIdx.x];
-  const int tx = wk.x % P.ntx, ty = wk.x / P.ntx;
-  const int gx0 = tx * kTile - kHalo, gy0 = ty * kTile - kHalo;
   constexpr int kPlane = kStageW * kStageW;
   // periodic indices: gx0 + lx lies in [-kHalo, nx + kTile + kHalo), one
   // wrap suffices when the grid is at least as wide as the staged region;
   // smaller grids take a full modulo
   const bool wide = P.nx >= kStageW && P.ny >= kStageW;
-  for (int e = threadIdx.x; e < 6 * kPlane; e += blockDim.x) {
-    const int c = e / kPlane;
-    const int r = e - c * kPlane;
-    const int ly = r / kStageW;
-    const int lx = r - ly * kStageW;
-    int gx = gx0 + lx, gy = gy0 + ly;
-    if (wide) {
-      gx += gx < 0 ? P.nx : (gx >= P.nx ? -P.nx : 0);
-      gy += gy < 0 ? P.ny : (gy >= P.ny ? -P.ny : 0);
-    } else {
-      gx %= P.nx;
-      gy %= P.ny;
-      gx += gx < 0 ? P.nx : 0;
-      gy += gy < 0 ? P.ny : 0;
-    }
-    // (the plane pointer indexed by a run-time c from the kernel's parameter
-    // space: a specialised kernel's copy of the parameters stays in registers)
-    tile_sm[TileGather<R>::pos(c, r)] =
-        __ldg(P_arg.yee[c] + static_cast<size_t>(gy) * P.nx + gx);
-  }
-  __syncthreads();
   Stage& stage = stage_all[threadIdx.x >> 5];
   int fill = 0;
   const PhotonOut pout = make_pout(P);
   Counts cnt;
-  const TileGather<R> gat{P, tile_sm, gx0, gy0};
-  for (int64_t base = wk.y; base < wk.z; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    PState<R> st;
-    if constexpr (kAos)
-      load_aos(P, i, i < wk.z, st);
-    else
-      load_state(P, i, i < wk.z, st);
-    advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, kAos>(
-        P, P.rkey, gat, i, st, stage, fill, pout, cnt);
+#pragma unroll 1
+  for (unsigned int item = blockIdx.x; item < items; item += gridDim.x) {
+    if (item != blockIdx.x) __syncthreads();  // (the tile before is still read)
+    const int4 wk = P.work[item];
+    const int tx = wk.x % P.ntx, ty = wk.x / P.ntx;
+    const int gx0 = tx * kTile - kHalo, gy0 = ty * kTile - kHalo;
+    for (int e = threadIdx.x; e < 6 * kPlane; e += blockDim.x) {
+      const int c = e / kPlane;
+      const int r = e - c * kPlane;
+      const int ly = r / kStageW;
+      const int lx = r - ly * kStageW;
+      int gx = gx0 + lx, gy = gy0 + ly;
+      if (wide) {
+        gx += gx < 0 ? P.nx : (gx >= P.nx ? -P.nx : 0);
+        gy += gy < 0 ? P.ny : (gy >= P.ny ? -P.ny : 0);
+      } else {
+        gx %= P.nx;
+        gy %= P.ny;
+        gx += gx < 0 ? P.nx : 0;
+        gy += gy < 0 ? P.ny : 0;
+      }
+      // (the plane pointer indexed by a run-time c from the kernel's parameter
+      // space: a specialised kernel's copy of the parameters stays in registers)
+      tile_sm[TileGather<R>::pos(c, r)] =
+          __ldg(P_arg.yee[c] + static_cast<size_t>(gy) * P.nx + gx);
+    }
+    __syncthreads();
+    const TileGather<R> gat{P, tile_sm, gx0, gy0};
+    for (int64_t base = wk.y; base < wk.z; base += blockDim.x) {
+      const int64_t i = base + threadIdx.x;
+      PState<R> st;
+      if constexpr (kAos)
+        load_aos(P, i, i < wk.z, st);
+      else
+        load_state(P, i, i < wk.z, st);
+      advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, kAos>(
+          P, P.rkey, gat, i, st, stage, fill, pout, cnt);
+    }
   }
   if (fill > 0) flush_stage(stage, fill, pout);
   flush_counts(cnt, P.counters);
@@ -1768,29 +1773,29 @@ bool std_config(const StepParams<R>& p, int dims) {
 }
 
 template <typename R, int CTRL, bool STD>
-cudaError_t launch_tiled_v(const StepParams<R>& p, int max_work, int block, cudaStream_t s) {
+cudaError_t launch_tiled_v(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
   // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
   cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kTileSmemBytes);
   if (e != cudaSuccess) return e;
-  k_push_emit_tiled<R, CTRL, STD><<<max_work, block, kTileSmemBytes, s>>>(p);
+  k_push_emit_tiled<R, CTRL, STD><<<grid, block, kTileSmemBytes, s>>>(p);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int max_work, int block,
+cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block,
                                    cudaStream_t s) {
   if (p.ang != nullptr) {
     if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
-      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, max_work, block, s);
-    return launch_tiled_v<R, 2, false>(p, max_work, block, s);
+      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, grid, block, s);
+    return launch_tiled_v<R, 2, false>(p, grid, block, s);
   }
   const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
-  if (ctrl) return launch_tiled_v<R, 1, false>(p, max_work, block, s);
+  if (ctrl) return launch_tiled_v<R, 1, false>(p, grid, block, s);
   if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
-    if (std_config(p, 2)) return launch_tiled_v<R, 0, true>(p, max_work, block, s);
-  return launch_tiled_v<R, 0, false>(p, max_work, block, s);
+    if (std_config(p, 2)) return launch_tiled_v<R, 0, true>(p, grid, block, s);
+  return launch_tiled_v<R, 0, false>(p, grid, block, s);
 }
 
 

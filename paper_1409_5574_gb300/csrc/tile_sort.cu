@@ -78,10 +78,6 @@ __device__ __forceinline__ unsigned int warp_claim(unsigned int* counter, int t,
   return slot;
 }
 
-// Binned gather: below this many particles per occupied tile the plain kernel
-// gathers from global memory (a tile's staging would not pay).
-constexpr unsigned int kBinSparse = 64;
-
 // Grid-stride over warps of 32 consecutive particles (every lane of a warp
 // takes the same number of iterations).
 template <typename R>
@@ -352,7 +348,9 @@ __global__ void __launch_bounds__(kBinThreads)
 template <bool SM>
 __global__ void __launch_bounds__(kBinThreads)
     k_bin_scatter(const BinGeom g, const float* __restrict__ x, const float* __restrict__ y,
-                  int64_t n, unsigned int* __restrict__ cursor, uint2* __restrict__ keys) {
+                  int64_t n, unsigned int* __restrict__ cursor,
+                  const unsigned int* __restrict__ gate, uint2* __restrict__ keys) {
+  if (*gate) return;
   extern __shared__ unsigned int s_tile[];
   const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
   if constexpr (SM) {
@@ -379,7 +377,8 @@ __global__ void __launch_bounds__(kBinThreads)
 // One block per tile: the slots of the tile's particles in cell order.
 __global__ void __launch_bounds__(kBinThreads)
     k_bin_cells(const uint2* __restrict__ keys, uint32_t* __restrict__ slot,
-                const unsigned int* __restrict__ starts) {
+                const unsigned int* __restrict__ starts, const unsigned int* __restrict__ gate) {
+  if (*gate) return;
   constexpr int kCells = kTile * kTile;
   static_assert(kCells == 2 * kBinThreads, "two cells per thread");
   __shared__ unsigned int s_cnt[kCells];
@@ -476,6 +475,7 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int
                             int num_sms, cudaStream_t s) {
   const int64_t n = p.n;
   const float *x = p.x, *y = p.y;
+  const unsigned int* gated = b.work_count + 1;  // (written by the scan)
   BinGeom g;
   g.nx = p.nx;
   g.ny = p.ny;
@@ -512,13 +512,13 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int
                                           gate ? kBinSparse : 0u);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (sm)
-    k_bin_scatter<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.cursor, b.keys);
+    k_bin_scatter<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.cursor, gated, b.keys);
   else
-    k_bin_scatter<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.cursor, b.keys);
+    k_bin_scatter<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.cursor, gated, b.keys);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_bin_cells<<<b.ntiles, kBinThreads, 0, s>>>(b.keys, b.slot, b.starts);
+  k_bin_cells<<<b.ntiles, kBinThreads, 0, s>>>(b.keys, b.slot, b.starts, gated);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_bin_pack<<<stream_grid(n, num_sms), 256, 0, s>>>(p, b.slot, b.work_count + 1, b.aos);
+  k_bin_pack<<<stream_grid(n, num_sms), 256, 0, s>>>(p, b.slot, gated, b.aos);
   return cudaGetLastError();
 }
 
