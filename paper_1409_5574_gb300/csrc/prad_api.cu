@@ -632,15 +632,25 @@ void free_sort(SortBuffers& b) {
 
 // The binned gather: a call takes it from kBinMinSteps steps and kBinMinWork
 // particle-steps on, and bins its particles again every kBinSteps steps (they
-// drift off the staged halo).  Measured, plain against binned, 4 steps and 8
-// steps in one launch: 2^20 particles in random order 649 against 289 and 1290
-// against 329 us, in cell order (whose plain gather hits L1) 188 against 249 and
-// 423 against 327 us; 2^17 particles, 8 steps: 194 against 146 and 79 against
-// 135 us.  Launches of fewer than kBinFused steps stage a tile for few
+// drift off the staged halo).  Measured, plain against binned, 8 steps in one
+// launch, 2^19 and 2^20 particles in random order 562 against 228 and 1114
+// against 341 us.  Launches of fewer than kBinFused steps stage a tile for few
 // particle-steps each: they take it from four times that work on, if the grid
-// holds kBinSparse particles per tile (8 one-step launches, 2^20 in cell order
-// 514 against 607 us, 16 of them 1207 against 1133; 40 of 2^18 spread over a 4096^2
+// holds kBinSparse particles per tile (40 launches of 2^18 spread over a 4096^2
 // grid 2134 against 2448).
+// In an order of cells the plain gather hits L1, and the binned one gains only
+// in long launches on many particles: 2^20 in one launch of 8 steps 268
+// against 318 us, of 16 steps 508 against 449; 2^21, 16 steps in launches of
+// one, two and four 1324 against 2040, 1158 against 1452 and 1059 against 1146
+// (in random order 4582 against 2086, 4570 and 4579 against 1503 and 1215; 8
+// steps in launches of one, 2^22 in cell order 1328 against 1777).  So launches of
+// fewer than kBinOrdered steps, and calls of less than 4 kBinMinWork, leave
+// particles to the plain kernel that follow an order of cells on the device's
+// count: more than half within near cells of the one before them, 16 for
+// launches of one step (break-even near a drift of 8 cells off that order, 2^21
+// 2123 against 2138 us, and an order of tiles alone, 1855 against 2159) and 4 for
+// the others (a drift of 1 to 3 cells: two steps a launch 1232 against 1474 and
+// 1524 against 1506).
 // Counting, scanning and the work list take 1 to 2 ns per tile of the grid, and
 // a sparse set pays for it in vain: a binning is tried only where kBinTileWork
 // particle-steps per tile follow, at 0.1 ns each (clumps) to 0.9 (2^19
@@ -650,6 +660,7 @@ void free_sort(SortBuffers& b) {
 constexpr int32_t kBinMinSteps = 8;
 constexpr int64_t kBinMinWork = int64_t(1) << 22;
 constexpr int kBinFused = 4;
+constexpr int kBinOrdered = 8;
 constexpr int32_t kBinSteps = 50;
 constexpr int64_t kBinTileWork = 64;
 
@@ -718,7 +729,7 @@ bool ensure_bins(prad_ctx* c, int64_t n, int ntiles) {
   if (cudaMalloc(&b.keys, np * sizeof(uint2)) != cudaSuccess ||
       cudaMalloc(&b.slot, np * sizeof(uint32_t)) != cudaSuccess ||
       cudaMalloc(&b.aos, np * 2 * sizeof(float4)) != cudaSuccess ||
-      cudaMalloc(&b.counts, sizeof(unsigned int) * ntiles) != cudaSuccess ||
+      cudaMalloc(&b.counts, sizeof(unsigned int) * (ntiles + 1)) != cudaSuccess ||
       cudaMalloc(&b.starts, sizeof(unsigned int) * (ntiles + 1)) != cudaSuccess ||
       cudaMalloc(&b.cursor, sizeof(unsigned int) * ntiles) != cudaSuccess ||
       cudaMalloc(&b.work, sizeof(int4) * mw) != cudaSuccess ||
@@ -751,27 +762,31 @@ bool can_bin(const prad_ctx* c) {
 // Whether a Yee launch takes the binned gather: FP32, table sampler, enough
 // particles and steps to pay for the binning, and no stream capture (whose
 // replays would share the scratch with other calls).  *gate: the particles may
-// turn out to be too sparse, so that the plain kernel stands behind each
-// launch.
-bool use_bins(prad_ctx* c, const StepParams<float>& p, int32_t nsteps, int sub, bool* gate) {
+// turn out to be too sparse, or (*near > 0) to follow an order of cells already,
+// so that the plain kernel stands behind each launch.
+bool use_bins(prad_ctx* c, const StepParams<float>& p, int32_t nsteps, int sub, bool* gate,
+              int* near) {
   const int64_t n = p.n;
   if (p.field_kind != PRAD_FIELD_YEE2D || !can_bin(c) || nsteps < kBinMinSteps ||
       n * nsteps < (sub < kBinFused ? 4 : 1) * kBinMinWork)
     return false;
   int ntx, nty;
   const int64_t ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
-  *gate = n < kBinSparse * ntiles;
-  if (*gate && sub < kBinFused) return false;
+  const bool sparse = n < kBinSparse * ntiles;
+  if (sparse && sub < kBinFused) return false;
+  *near = sub == 1 ? 16 : sub < kBinOrdered || n * nsteps < 4 * kBinMinWork ? 4 : 0;
+  *gate = sparse || *near > 0;
   if (n * std::min(nsteps, kBinSteps) < kBinTileWork * ntiles) return false;
   return !capturing(c);
 }
 
-// Blocks of a tiled launch of at most mw work items: eight for every resident
-// one (three per SM), each taking more than one item only where there are
-// more.  (A block per possible item, most of them empty where the particles
-// fill a part of the grid, costs about 0.9 ns each.)
-int tiled_grid(int64_t mw, int num_sms) {
-  return static_cast<int>(std::min<int64_t>(mw, 8 * 3 * static_cast<int64_t>(num_sms)));
+// Blocks of a tiled launch of at most mw work items: per resident one (three
+// per SM) eight, or two where a gate may leave the launch without work, each
+// taking more than one item only where there are more.  (A block per possible
+// item, most of them empty where the particles fill a part of the grid, costs
+// about 0.9 ns each; a launch of eight without work 5 us, of two 2.)
+int tiled_grid(int64_t mw, int num_sms, int per = 8) {
+  return static_cast<int>(std::min<int64_t>(mw, per * 3 * static_cast<int64_t>(num_sms)));
 }
 
 // Scratch for the sort: max_particles copies of the 7 state arrays and the
@@ -825,7 +840,7 @@ int bin_fp32(prad_ctx* c, const StepParams<float>& p, int chunk) {
   c->bins_sorted = true;
   BinBuffers b = c->bins;
   b.ntiles = ntiles;
-  CK(c, launch_tile_bin(p, b, chunk, false, c->num_sms, c->stream));
+  CK(c, launch_tile_bin(p, b, chunk, false, 0, c->num_sms, c->stream));
   return PRAD_OK;
 }
 
@@ -878,14 +893,17 @@ int spec_for(prad_ctx* c, const StepParams<float>& p, bool tiled, const SpecFn**
 // A Yee push of particles that stay in the caller's order: every kBinSteps
 // steps the state is copied in the order of tiles and cells, the launches in
 // between run the tile-staged kernel on the copy, and it is written back.
-// gate: where the particles turn out to be sparse nothing is copied, the tile
-// work is empty and the plain kernel (grid, block) behind each launch runs
-// instead (a word on the device decides, nothing is read back).  A specialised
+// gate: where the particles turn out to be sparse or (near) in an order of cells
+// nothing is copied, the tile work is empty and the plain kernel (grid, block)
+// behind each launch runs instead (a word on the device decides, nothing is read
+// back; each of the two starts while the other drains: 16 one-step launches of
+// 2^21 in cell order 1386 us, 1460 without the overlap, 1320 plain).  A specialised
 // context compiles one kernel for a call: the tiled one (1.06 times the
 // compiled-in one's speed), or with a gate the plain one (plain).
 // *taken: false if the scratch cannot be had, and nothing was launched.
 int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int32_t nsteps,
-                int sub, bool gate, const SpecFn* plain, int grid, int block, bool* taken) {
+                int sub, bool gate, int near, const SpecFn* plain, int grid, int block,
+                bool* taken) {
   // (one lock for the scratch and everything that is launched on it)
   std::lock_guard<std::mutex> lk(c->bin_mu);
   int ntx, nty;
@@ -905,9 +923,9 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   const int rc = gate ? PRAD_OK : spec_for(c, p, true, &spec);
   if (rc != PRAD_OK) return rc;
   const int chunk = chunk_of(p.n, sub < nsteps ? sub : nsteps, c->num_sms);
-  const int tgrid = tiled_grid(max_work_items(p.n, ntiles, chunk), c->num_sms);
+  const int tgrid = tiled_grid(max_work_items(p.n, ntiles, chunk), c->num_sms, gate ? 2 : 8);
   for (int32_t done = 0; done < nsteps;) {
-    CK(c, launch_tile_bin(p, b, chunk, gate, c->num_sms, c->stream));
+    CK(c, launch_tile_bin(p, b, chunk, gate, near, c->num_sms, c->stream));
     const int32_t end = done + kBinSteps;
     while (done < nsteps && done < end) {
       const int32_t m = (nsteps - done) < sub ? (nsteps - done) : sub;
@@ -915,18 +933,18 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
       p.nsub = m;
       p.gate = nullptr;
       if (spec) {
-        CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
+        CK(c, spec_launch(spec, p, tgrid, 256, c->stream, gate));
         ++c->spec_launches;
       } else {
-        CK(c, launch_push_emit_tiled<float>(p, tgrid, 256, c->stream));
+        CK(c, launch_push_emit_tiled<float>(p, tgrid, 256, c->stream, gate));
       }
       p.gate = b.work_count + 1;
       if (gate && plain) {
-        CK(c, spec_launch(plain, p, grid, block, c->stream, false));
+        CK(c, spec_launch(plain, p, grid, block, c->stream, true));
         ++c->spec_launches;
       } else if (gate) {
         CK(c, launch_push_emit<float>(p, p.field_kind, c->cfg.sampler, grid, block, c->stream,
-                                      false));
+                                      true));
       }
       done += m;
     }
@@ -992,7 +1010,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
           CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
           ++c->spec_launches;
         } else {
-          CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream));
+          CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream, false));
         }
         CK(c, launch_tile_unsort(p, c->bins, static_cast<float*>(pp->w), pp->pid, c->num_sms,
                                  c->stream));
@@ -1002,7 +1020,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         p.work = c->sort.work;
         p.work_count = c->sort.work_count;
         const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms);
-        CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream));
+        CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream, false));
       }
       done += m;
     }
@@ -1037,11 +1055,13 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
   if constexpr (sizeof(R) == 4) {
     p.nsub = sub_eff;
     bool gate = false;
-    if (use_bins(c, p, nsteps, sub, &gate)) {
+    int near = 0;
+    if (use_bins(c, p, nsteps, sub, &gate, &near)) {
       bool taken = false;
       int rc = gate ? spec_for(c, p, false, &spec) : PRAD_OK;
       if (rc == PRAD_OK)
-        rc = push_binned(c, p, pp, nsteps, sub, gate, spec, gate ? grid_of() : 0, block, &taken);
+        rc = push_binned(c, p, pp, nsteps, sub, gate, near, spec, gate ? grid_of() : 0, block,
+                         &taken);
       if (rc != PRAD_OK || taken) return rc;
     }
     const int rc = spec_for(c, p, false, &spec);

@@ -210,7 +210,7 @@ struct BinBuffers {
   uint2* keys;
   uint32_t* slot;
   float4* aos;                // two per particle
-  unsigned int* counts;       // per tile
+  unsigned int* counts;       // per tile, then particles near the one before them
   unsigned int* starts;       // per tile + 1
   unsigned int* cursor;       // per tile
   int4* work;
@@ -269,19 +269,21 @@ cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
                           uint32_t* out, int64_t n, cudaStream_t s);
 template <typename R>
-cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block,
-                                   cudaStream_t s);
+cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block, cudaStream_t s,
+                                   bool pdl);
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,
                              int nx, int ny, double x0, double y0, double inv_dx,
                              double inv_dy, int chunk, cudaStream_t s);
 // The state of the p.n particles of p into b.aos in the order of their tiles
 // and cells, and the work list (chunks of at most `chunk` particles of one
-// tile); gate: sparse particles leave that to the plain kernel.
+// tile); sparse: particles that are sparse leave that to the plain kernel;
+// near > 0: so do particles of which more than half lie within near cells of
+// the one before them.
 // launch_tile_unbin writes the state back to where it came from,
 // launch_tile_unsort in its new order, with the weights and ids.
-cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool gate,
-                            int num_sms, cudaStream_t s);
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool sparse,
+                            int near, int num_sms, cudaStream_t s);
 cudaError_t launch_tile_unsort(const StepParams<float>& p, const BinBuffers& b, float* w,
                                uint32_t* pid, int num_sms, cudaStream_t s);
 cudaError_t launch_tile_unbin(const StepParams<float>& p, const BinBuffers& b, int num_sms,
@@ -362,8 +364,7 @@ cudaError_t spec_get(SpecCache* c, int device, const StepParams<float>& p, const
                      const SpecFn** out, char* msg, size_t msg_len);
 int spec_occupancy(const SpecFn* f, int block);
 // grid blocks of block threads; the tiled kernel gets its tile's dynamic
-// shared memory.  pdl: as launch_push_emit's (not for the tiled kernel, which
-// does not wait for the launch before itself)
+// shared memory.  pdl: as launch_push_emit's
 cudaError_t spec_launch(const SpecFn* f, const StepParams<float>& p, int grid, int block,
                         cudaStream_t s, bool pdl);
 // Whether a launch with these parameters runs a specialisable variant (FP32

@@ -1695,6 +1695,8 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   const StepParams<R>& P = P_arg;
 #endif
   constexpr bool kAos = sizeof(R) == 4;
+  pdl_wait();
+  pdl_trigger();
   const unsigned int items = *P.work_count;
   if (blockIdx.x >= items) return;
   extern __shared__ __align__(16) float tile_sm[];
@@ -1772,40 +1774,14 @@ bool std_config(const StepParams<R>& p, int dims) {
          p.abs_q == R(1);
 }
 
-template <typename R, int CTRL, bool STD>
-cudaError_t launch_tiled_v(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
-  // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
-  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kTileSmemBytes);
-  if (e != cudaSuccess) return e;
-  k_push_emit_tiled<R, CTRL, STD><<<grid, block, kTileSmemBytes, s>>>(p);
-  return cudaGetLastError();
-}
-
-template <typename R>
-cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block,
-                                   cudaStream_t s) {
-  if (p.ang != nullptr) {
-    if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
-      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, grid, block, s);
-    return launch_tiled_v<R, 2, false>(p, grid, block, s);
-  }
-  const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
-  if (ctrl) return launch_tiled_v<R, 1, false>(p, grid, block, s);
-  if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
-    if (std_config(p, 2)) return launch_tiled_v<R, 0, true>(p, grid, block, s);
-  return launch_tiled_v<R, 0, false>(p, grid, block, s);
-}
-
-
 // pdl: the launch may begin before the stream's earlier work is done (pdl_wait).
 template <typename R>
 void launch_one(void (*kernel)(const StepParams<R>), const StepParams<R>& p, int grid, int block,
-                cudaStream_t s, bool pdl) {
+                cudaStream_t s, bool pdl, size_t dyn_smem = 0) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(static_cast<unsigned>(block));
+  cfg.dynamicSmemBytes = dyn_smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1813,6 +1789,32 @@ void launch_one(void (*kernel)(const StepParams<R>), const StepParams<R>& p, int
   cfg.attrs = at;
   cfg.numAttrs = pdl ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kernel, p);  // (the caller reads the last error)
+}
+
+template <typename R, int CTRL, bool STD>
+cudaError_t launch_tiled_v(const StepParams<R>& p, int grid, int block, cudaStream_t s, bool pdl) {
+  // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
+  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kTileSmemBytes);
+  if (e != cudaSuccess) return e;
+  launch_one(k_push_emit_tiled<R, CTRL, STD>, p, grid, block, s, pdl, kTileSmemBytes);
+  return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block, cudaStream_t s,
+                                   bool pdl) {
+  if (p.ang != nullptr) {
+    if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
+      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, grid, block, s, pdl);
+    return launch_tiled_v<R, 2, false>(p, grid, block, s, pdl);
+  }
+  const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
+  if (ctrl) return launch_tiled_v<R, 1, false>(p, grid, block, s, pdl);
+  if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
+    if (std_config(p, 2)) return launch_tiled_v<R, 0, true>(p, grid, block, s, pdl);
+  return launch_tiled_v<R, 0, false>(p, grid, block, s, pdl);
 }
 
 template <typename R, int FIELD, int SAMP, int PF, int CTRL>
@@ -2070,8 +2072,10 @@ template cudaError_t launch_push_emit<float>(const StepParams<float>&, int, int,
                                             cudaStream_t, bool);
 template cudaError_t launch_push_emit<double>(const StepParams<double>&, int, int, int, int,
                                              cudaStream_t, bool);
-template cudaError_t launch_push_emit_tiled<float>(const StepParams<float>&, int, int, cudaStream_t);
-template cudaError_t launch_push_emit_tiled<double>(const StepParams<double>&, int, int, cudaStream_t);
+template cudaError_t launch_push_emit_tiled<float>(const StepParams<float>&, int, int, cudaStream_t,
+                                                   bool);
+template cudaError_t launch_push_emit_tiled<double>(const StepParams<double>&, int, int,
+                                                    cudaStream_t, bool);
 template cudaError_t launch_eval_sampler<float>(const StepParams<float>&, const uint32_t*, float*, float*, int64_t, cudaStream_t);
 template cudaError_t launch_eval_sampler<double>(const StepParams<double>&, const uint32_t*, double*, double*, int64_t, cudaStream_t);
 

@@ -112,12 +112,14 @@ __device__ __forceinline__ unsigned int warp_inclusive(unsigned int v, int lane)
 }
 
 // sparse > 0 (binned gather): with fewer than `sparse` particles per occupied
-// tile there is no tile work, and the gate lets the plain kernel run instead.
+// tile there is no tile work, and the gate lets the plain kernel run instead;
+// so too with at least `ordered` > 0 particles near the one before them
+// (k_bin_count's last counter).
 __global__ void __launch_bounds__(kScanThreads)
     k_tile_scan(const unsigned int* __restrict__ counts, int ntiles,
                 unsigned int* __restrict__ starts, unsigned int* __restrict__ cursor,
                 int4* __restrict__ work, unsigned int* __restrict__ work_count,
-                unsigned int chunk, unsigned int sparse) {
+                unsigned int chunk, unsigned int sparse, unsigned int ordered) {
   constexpr int kWarps = kScanThreads / 32;
   __shared__ unsigned int s_sum[kWarps], s_chunks[kWarps], s_used[kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -148,7 +150,8 @@ __global__ void __launch_bounds__(kScanThreads)
     s_chunks[lane] = ib - b;
     if (lane == 31) {
       starts[ntiles] = ia;
-      const bool none = sparse != 0u && ia < static_cast<uint64_t>(sparse) * tiles;
+      const bool none = (sparse != 0u && ia < static_cast<uint64_t>(sparse) * tiles) ||
+                        (ordered != 0u && counts[ntiles] >= ordered);
       work_count[0] = none ? 0u : ib;
       work_count[1] = none ? 1u : 0u;
     }
@@ -324,12 +327,31 @@ __device__ __forceinline__ void bin_count_range(const BinGeom& g, const float* _
   }
 }
 
+// near > 0: how many particles lie within that many cells, in x and in y, of
+// the one before them in the caller's order (a warp's first counts as one) is
+// added to counts[g.ntiles]: in an order of cells nearly all, in a random one
+// few, and the plain gather's loads meet in L1 where they do.
 template <bool SM>
 __global__ void __launch_bounds__(kBinThreads)
     k_bin_count(const BinGeom g, const float* __restrict__ x, const float* __restrict__ y,
-                int64_t n, unsigned int* __restrict__ counts) {
+                int64_t n, unsigned int* __restrict__ counts, int near) {
   extern __shared__ unsigned int s_tile[];
   const int64_t lo = n * blockIdx.x / gridDim.x, hi = n * (blockIdx.x + 1) / gridDim.x;
+  if (near > 0) {
+    const int lane = threadIdx.x & 31;
+    unsigned int mine = 0u;
+#pragma unroll 4
+    for (int64_t w0 = lo + (threadIdx.x & ~31); w0 < hi; w0 += kBinThreads) {
+      const int64_t i = w0 + lane;
+      const int2 c = i < hi ? cell_xy(x[i], y[i], g.nx, g.ny, g.x0, g.y0, g.inv_dx, g.inv_dy)
+                            : make_int2(0, 0);
+      const int px = __shfl_up_sync(0xffffffffu, c.x, 1);
+      const int py = __shfl_up_sync(0xffffffffu, c.y, 1);
+      mine += i < hi && (lane == 0 || (abs(c.x - px) <= near && abs(c.y - py) <= near));
+    }
+    mine = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0 && mine) atomicAdd(counts + g.ntiles, mine);
+  }
   if constexpr (SM) {
     for (int t = threadIdx.x; t < g.ntiles; t += kBinThreads) s_tile[t] = 0u;
     __syncthreads();
@@ -471,8 +493,8 @@ int stream_grid(int64_t n, int num_sms) {
 
 }  // namespace
 
-cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool gate,
-                            int num_sms, cudaStream_t s) {
+cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int chunk, bool sparse,
+                            int near, int num_sms, cudaStream_t s) {
   const int64_t n = p.n;
   const float *x = p.x, *y = p.y;
   const unsigned int* gated = b.work_count + 1;  // (written by the scan)
@@ -485,7 +507,7 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int
   g.y0 = p.y0;
   g.inv_dx = p.inv_dx;
   g.inv_dy = p.inv_dy;
-  cudaError_t e = cudaMemsetAsync(b.counts, 0, sizeof(unsigned int) * b.ntiles, s);
+  cudaError_t e = cudaMemsetAsync(b.counts, 0, sizeof(unsigned int) * (b.ntiles + 1), s);
   if (e != cudaSuccess) return e;
   const bool sm = b.ntiles <= kBinTiles;
   const size_t dyn = sm ? sizeof(unsigned int) * b.ntiles : 0;
@@ -503,13 +525,14 @@ cudaError_t launch_tile_bin(const StepParams<float>& p, const BinBuffers& b, int
   const int64_t want = (n + 2047) / 2048;
   const int grid = static_cast<int>(want < 3 * num_sms ? want : 3 * num_sms);
   if (sm)
-    k_bin_count<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.counts);
+    k_bin_count<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.counts, near);
   else
-    k_bin_count<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.counts);
+    k_bin_count<false><<<grid, kBinThreads, 0, s>>>(g, x, y, n, b.counts, near);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_tile_scan<<<1, kScanThreads, 0, s>>>(b.counts, b.ntiles, b.starts, b.cursor, b.work,
                                           b.work_count, static_cast<unsigned int>(chunk),
-                                          gate ? kBinSparse : 0u);
+                                          sparse ? kBinSparse : 0u,
+                                          near > 0 ? static_cast<unsigned int>(n / 2 + 1) : 0u);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (sm)
     k_bin_scatter<true><<<grid, kBinThreads, dyn, s>>>(g, x, y, n, b.cursor, gated, b.keys);
@@ -549,7 +572,8 @@ cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuff
                                          R(inv_dx), R(inv_dy), b.counts);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   k_tile_scan<<<1, kScanThreads, 0, s>>>(b.counts, b.ntiles, b.starts, b.cursor, b.work,
-                                          b.work_count, static_cast<unsigned int>(chunk), 0u);
+                                          b.work_count, static_cast<unsigned int>(chunk), 0u,
+                                          0u);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   Arrays7<R> srcp, dstp;
   for (int k = 0; k < 7; ++k) {

@@ -57,6 +57,11 @@ CASES = {
     "sparse, specialised": (4100, 4129, 524_301, 4000, 4000, None, 0.0, 9, 8, dict(specialize=True)),
     "clump, specialised": (4100, 4129, 524_301, 60, 70, None, 0.0, 9, 8, dict(specialize=True)),
     "dense, specialised": (256, 250, 2_097_152, 256, 250, None, 0.0, 9, 9, dict(specialize=True)),
+    "rows of cells, one step": (300, 280, 2_097_152, 300, 280, "rows", 0.0, 9, 1, {}),
+    "cells, drifted, one step": (300, 280, 2_097_152, 300, 280, "cells", 40.0, 9, 1, {}),
+    "cells, specialised": (2050, 2049, 2_097_152, 500, 500, "cells", 0.3, 9, 4, dict(specialize=True)),
+    "random, specialised": (500, 490, 2_097_152, 500, 490, None, 0.0, 9, 4, dict(specialize=True)),
+    "cells, short": (96, 130, 524_301, 96, 130, "cells", 0.0, 9, 9, {}),
     "more tiles than work": (8200, 8190, 524_301, 60, 70, None, 0.0, 8, 8, {}),
 }
 
