@@ -648,9 +648,9 @@ void free_sort(SortBuffers& b) {
 // particles to the plain kernel that follow an order of cells on the device's
 // count: more than half within near cells of the one before them, 16 for
 // launches of one step (break-even near a drift of 8 cells off that order, 2^21
-// 2123 against 2138 us, and an order of tiles alone, 1855 against 2159) and 4 for
+// 2123 against 2138 us, and an order of tiles alone, 1855 against 2159) and 3 for
 // the others (a drift of 1 to 3 cells: two steps a launch 1232 against 1474 and
-// 1524 against 1506).
+// 1524 against 1506; 2^20, 8 steps in one, a drift of 3 cells 399 against 325).
 // Counting, scanning and the work list take 1 to 2 ns per tile of the grid, and
 // a sparse set pays for it in vain: a binning is tried only where kBinTileWork
 // particle-steps per tile follow, at 0.1 ns each (clumps) to 0.9 (2^19
@@ -774,7 +774,7 @@ bool use_bins(prad_ctx* c, const StepParams<float>& p, int32_t nsteps, int sub, 
   const int64_t ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
   const bool sparse = n < kBinSparse * ntiles;
   if (sparse && sub < kBinFused) return false;
-  *near = sub == 1 ? 16 : sub < kBinOrdered || n * nsteps < 4 * kBinMinWork ? 4 : 0;
+  *near = sub == 1 ? 16 : sub < kBinOrdered || n * nsteps < 4 * kBinMinWork ? 3 : 0;
   *gate = sparse || *near > 0;
   if (n * std::min(nsteps, kBinSteps) < kBinTileWork * ntiles) return false;
   return !capturing(c);
