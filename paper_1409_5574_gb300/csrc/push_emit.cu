@@ -707,6 +707,8 @@ __device__ __forceinline__ void flush_stage(ST& st, int fill, const PhotonOut& o
   if (lane == 0) base = atomicAdd(o.cursor, static_cast<unsigned long long>(fill));
   base = __shfl_sync(0xffffffffu, base, 0);
   __syncwarp();
+  // (two rounds at most, rolled: 15 ms less for a kernel compiled at run time)
+#pragma unroll 1
   for (int r = lane; r < fill; r += 32) {
     const unsigned long long slot = base + static_cast<unsigned>(r);
     if (slot < static_cast<unsigned long long>(o.cap)) {
@@ -1039,15 +1041,22 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
   (void)dtn32; (void)eps32; (void)cn32;
   // Two steps per iteration on the analytic fields in FP32 (the end of one
   // overlaps the start of the next; 2^22 electrons, 100 steps: 4123 against
-  // 4007 us, with run-time specialised constants 3607 against 3567 on a late
-  // stretch).  Three or more outgrow the registers; the Yee step is too long
-  // for two (2^22 sorted electrons 8331 against 8370 us), and so is the
-  // batched kernel's, whose parameters take registers (64 ensembles 3690
-  // against 3712 us; it and the control kernels stage by field).
+  // 4007 us; with the angular spread 4904 against 4860, 2^20 1273 against 1260).
+  // Three or more outgrow the registers; the Yee step is too long for two (2^22
+  // sorted electrons 8331 against 8370 us), and so is the batched kernel's, whose
+  // parameters take registers (64 ensembles 3690 against 3712 us; it and the
+  // control kernels without the spread share the staging by field).  Kernels
+  // compiled at run time keep one: a second step gains 190 us per 100 steps of
+  // 2^24 electrons (15510 against 15710), and costs the context's first call 75
+  // ms of compilation, which a run of 4000 steps does not win back.
+#ifdef PRAD_SPEC
+  constexpr int kUnroll = 1;
+#else
   constexpr int kUnroll = sizeof(R) == 4 && FIELD != PRAD_FIELD_YEE2D &&
                                   !std::is_same<ST, PhotonStageSoA>::value
                               ? 2
                               : 1;
+#endif
 #pragma unroll kUnroll
   for (int s = 0; s < nsub; ++s) {
     const uint32_t step = static_cast<uint32_t>(P.t0 + s);
