@@ -646,11 +646,12 @@ void free_sort(SortBuffers& b) {
 // steps in launches of one, 2^22 in cell order 1328 against 1777).  So launches of
 // fewer than kBinOrdered steps, and calls of less than 4 kBinMinWork, leave
 // particles to the plain kernel that follow an order of cells on the device's
-// count: more than half within near cells of the one before them, 16 for
-// launches of one step (break-even near a drift of 8 cells off that order, 2^21
-// 2123 against 2138 us, and an order of tiles alone, 1855 against 2159) and 3 for
-// the others (a drift of 1 to 3 cells: two steps a launch 1232 against 1474 and
-// 1524 against 1506; 2^20, 8 steps in one, a drift of 3 cells 399 against 325).
+// count: more than half within near cells of the one before them, 8 for launches
+// of one step (a drift of 3 cells off that order, 2^22: 3329 against 3425 us; of
+// 8 cells, binned, 4264 against 3423, 2^21 2123 against 2138) and 3 for the
+// others (a drift of 1 and of 3 cells, 2^21, two steps a launch: 1232 against
+// 1474 and, binned, 1524 against 1506; 2^20, 8 steps in one, 3 cells: binned, 399
+// against 325).
 // Counting, scanning and the work list take 1 to 2 ns per tile of the grid, and
 // a sparse set pays for it in vain: a binning is tried only where kBinTileWork
 // particle-steps per tile follow, at 0.1 ns each (clumps) to 0.9 (2^19
@@ -774,19 +775,18 @@ bool use_bins(prad_ctx* c, const StepParams<float>& p, int32_t nsteps, int sub, 
   const int64_t ntiles = tile_counts(p.nx, p.ny, &ntx, &nty);
   const bool sparse = n < kBinSparse * ntiles;
   if (sparse && sub < kBinFused) return false;
-  *near = sub == 1 ? 16 : sub < kBinOrdered || n * nsteps < 4 * kBinMinWork ? 3 : 0;
+  *near = sub == 1 ? 8 : sub < kBinOrdered || n * nsteps < 4 * kBinMinWork ? 3 : 0;
   *gate = sparse || *near > 0;
   if (n * std::min(nsteps, kBinSteps) < kBinTileWork * ntiles) return false;
   return !capturing(c);
 }
 
-// Blocks of a tiled launch of at most mw work items: per resident one (three
-// per SM) eight, or two where a gate may leave the launch without work, each
-// taking more than one item only where there are more.  (A block per possible
-// item, most of them empty where the particles fill a part of the grid, costs
-// about 0.9 ns each; a launch of eight without work 5 us, of two 2.)
-int tiled_grid(int64_t mw, int num_sms, int per = 8) {
-  return static_cast<int>(std::min<int64_t>(mw, per * 3 * static_cast<int64_t>(num_sms)));
+// Blocks of a tiled launch of at most mw work items: one each, or behind a gate,
+// where the launch may find no work, two per resident block (three per SM),
+// which take the items in turn.  (A block without an item costs about 0.9 ns, a
+// launch of two per resident block without work 2 us.)
+int tiled_grid(int64_t mw, int num_sms, bool gate) {
+  return static_cast<int>(gate ? std::min<int64_t>(mw, 6 * static_cast<int64_t>(num_sms)) : mw);
 }
 
 // Scratch for the sort: max_particles copies of the 7 state arrays and the
@@ -923,7 +923,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
   const int rc = gate ? PRAD_OK : spec_for(c, p, true, &spec);
   if (rc != PRAD_OK) return rc;
   const int chunk = chunk_of(p.n, sub < nsteps ? sub : nsteps, c->num_sms);
-  const int tgrid = tiled_grid(max_work_items(p.n, ntiles, chunk), c->num_sms, gate ? 2 : 8);
+  const int tgrid = tiled_grid(max_work_items(p.n, ntiles, chunk), c->num_sms, gate);
   for (int32_t done = 0; done < nsteps;) {
     CK(c, launch_tile_bin(p, b, chunk, gate, near, c->num_sms, c->stream));
     const int32_t end = done + kBinSteps;
@@ -933,7 +933,7 @@ int push_binned(prad_ctx* c, StepParams<float> p, const prad_particles* pp, int3
       p.nsub = m;
       p.gate = nullptr;
       if (spec) {
-        CK(c, spec_launch(spec, p, tgrid, 256, c->stream, gate));
+        CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
         ++c->spec_launches;
       } else {
         CK(c, launch_push_emit_tiled<float>(p, tgrid, 256, c->stream, gate));
@@ -1005,7 +1005,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         p.aos = c->bins.aos;
         p.work = c->bins.work;
         p.work_count = c->bins.work_count;
-        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms);
+        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms, false);
         if (spec) {
           CK(c, spec_launch(spec, p, tgrid, 256, c->stream, false));
           ++c->spec_launches;
@@ -1019,7 +1019,7 @@ int push_emit_t(prad_ctx* c, const prad_particles* pp, int64_t n,
         if (rc != PRAD_OK) return rc;
         p.work = c->sort.work;
         p.work_count = c->sort.work_count;
-        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms);
+        const int tgrid = tiled_grid(max_work_items(n, ntx * nty, chunk), c->num_sms, false);
         CK(c, launch_push_emit_tiled<R>(p, tgrid, 256, c->stream, false));
       }
       done += m;

@@ -268,9 +268,11 @@ cudaError_t launch_eval_sampler(const StepParams<R>& p, const uint32_t* words,
                                 R* x_out, R* g_out, int64_t n, cudaStream_t s);
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,
                           uint32_t* out, int64_t n, cudaStream_t s);
+// gated (FP32): the launch may find no work, has a bounded grid whose blocks
+// take several items each, and may begin while the one before it drains
 template <typename R>
 cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block, cudaStream_t s,
-                                   bool pdl);
+                                   bool gated);
 template <typename R>
 cudaError_t launch_tile_sort(R* arr[7], uint32_t* pid, int64_t n, const SortBuffers& b,
                              int nx, int ny, double x0, double y0, double inv_dx,

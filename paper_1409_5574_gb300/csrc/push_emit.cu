@@ -707,8 +707,11 @@ __device__ __forceinline__ void flush_stage(ST& st, int fill, const PhotonOut& o
   if (lane == 0) base = atomicAdd(o.cursor, static_cast<unsigned long long>(fill));
   base = __shfl_sync(0xffffffffu, base, 0);
   __syncwarp();
-  // (two rounds at most, rolled: 15 ms less for a kernel compiled at run time)
+  // (two rounds at most; rolled where the kernel is compiled at run time: 15 ms
+  // less of that)
+#ifdef PRAD_SPEC
 #pragma unroll 1
+#endif
   for (int r = lane; r < fill; r += 32) {
     const unsigned long long slot = base + static_cast<unsigned>(r);
     if (slot < static_cast<unsigned long long>(o.cap)) {
@@ -1704,8 +1707,10 @@ int batch_max_blocks_per_sm(int block, int sampler, bool ctrl, bool std_cfg) {
 // (+ halo, periodic) in shared memory with coalesced row loads, then runs the
 // same per-particle path with the shared-memory gather.
 // ---------------------------------------------------------------------------
-// FP32: the state is the binned copy (P.aos).
-template <typename R, int CTRL, bool STD = false>
+// FP32: the state is the binned copy (P.aos).  LOOP: a block takes every
+// gridDim.x-th item (launches behind a gate, whose grid is bounded; as a loop
+// the kernel is 2.7% slower, so the others take one item per block).
+template <typename R, int CTRL, bool STD = false, bool LOOP = false>
 __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> P_arg) {
 #ifdef PRAD_SPEC
   const StepParams<R> P = spec_params(P_arg);
@@ -1713,8 +1718,10 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   const StepParams<R>& P = P_arg;
 #endif
   constexpr bool kAos = sizeof(R) == 4;
-  pdl_wait();
-  pdl_trigger();
+  if constexpr (LOOP) {
+    pdl_wait();
+    pdl_trigger();
+  }
   const unsigned int items = *P.work_count;
   if (blockIdx.x >= items) return;
   extern __shared__ __align__(16) float tile_sm[];
@@ -1729,9 +1736,8 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
   int fill = 0;
   const PhotonOut pout = make_pout(P);
   Counts cnt;
-#pragma unroll 1
-  for (unsigned int item = blockIdx.x; item < items; item += gridDim.x) {
-    if (item != blockIdx.x) __syncthreads();  // (the tile before is still read)
+  unsigned int item = blockIdx.x;
+  do {
     const int4 wk = P.work[item];
     const int tx = wk.x % P.ntx, ty = wk.x / P.ntx;
     const int gx0 = tx * kTile - kHalo, gy0 = ty * kTile - kHalo;
@@ -1767,7 +1773,11 @@ __global__ void __launch_bounds__(256, 3) k_push_emit_tiled(const StepParams<R> 
       advance_particle<R, PRAD_FIELD_YEE2D, PRAD_SAMPLER_TABLE, 0, CTRL, STD, false, 0, kAos>(
           P, P.rkey, gat, i, st, stage, fill, pout, cnt);
     }
-  }
+    if constexpr (LOOP) {
+      item += gridDim.x;
+      if (item < items) __syncthreads();  // (the tile is still read)
+    }
+  } while (LOOP && item < items);
   if (fill > 0) flush_stage(stage, fill, pout);
   flush_counts(cnt, P.counters);
 }
@@ -1809,30 +1819,37 @@ void launch_one(void (*kernel)(const StepParams<R>), const StepParams<R>& p, int
   (void)cudaLaunchKernelEx(&cfg, kernel, p);  // (the caller reads the last error)
 }
 
-template <typename R, int CTRL, bool STD>
-cudaError_t launch_tiled_v(const StepParams<R>& p, int grid, int block, cudaStream_t s, bool pdl) {
+template <typename R, int CTRL, bool STD, bool LOOP>
+cudaError_t launch_tiled_v(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
   // dynamic tile (46.5 KB) + static photon staging exceed the 48 KB default
-  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD>,
+  cudaError_t e = cudaFuncSetAttribute(k_push_emit_tiled<R, CTRL, STD, LOOP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kTileSmemBytes);
   if (e != cudaSuccess) return e;
-  launch_one(k_push_emit_tiled<R, CTRL, STD>, p, grid, block, s, pdl, kTileSmemBytes);
+  launch_one(k_push_emit_tiled<R, CTRL, STD, LOOP>, p, grid, block, s, LOOP, kTileSmemBytes);
   return cudaGetLastError();
+}
+
+template <typename R, bool LOOP>
+cudaError_t launch_tiled_l(const StepParams<R>& p, int grid, int block, cudaStream_t s) {
+  if (p.ang != nullptr) {
+    if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
+      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true, LOOP>(p, grid, block, s);
+    return launch_tiled_v<R, 2, false, LOOP>(p, grid, block, s);
+  }
+  const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
+  if (ctrl) return launch_tiled_v<R, 1, false, LOOP>(p, grid, block, s);
+  if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
+    if (std_config(p, 2)) return launch_tiled_v<R, 0, true, LOOP>(p, grid, block, s);
+  return launch_tiled_v<R, 0, false, LOOP>(p, grid, block, s);
 }
 
 template <typename R>
 cudaError_t launch_push_emit_tiled(const StepParams<R>& p, int grid, int block, cudaStream_t s,
-                                   bool pdl) {
-  if (p.ang != nullptr) {
-    if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 2>)
-      if (std_config(p, 2) && one_trial(p)) return launch_tiled_v<R, 2, true>(p, grid, block, s, pdl);
-    return launch_tiled_v<R, 2, false>(p, grid, block, s, pdl);
-  }
-  const bool ctrl = p.ntry > 1 || p.sel_q < R(1) || p.diag != 0;
-  if (ctrl) return launch_tiled_v<R, 1, false>(p, grid, block, s, pdl);
-  if constexpr (kHasStd<R, PRAD_FIELD_YEE2D, 0>)
-    if (std_config(p, 2)) return launch_tiled_v<R, 0, true>(p, grid, block, s, pdl);
-  return launch_tiled_v<R, 0, false>(p, grid, block, s, pdl);
+                                   bool gated) {
+  if constexpr (sizeof(R) == 4)
+    if (gated) return launch_tiled_l<R, true>(p, grid, block, s);
+  return launch_tiled_l<R, false>(p, grid, block, s);
 }
 
 template <typename R, int FIELD, int SAMP, int PF, int CTRL>
