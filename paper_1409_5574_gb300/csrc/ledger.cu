@@ -157,8 +157,9 @@ __device__ __forceinline__ uint32_t bit_of(uint32_t s) {
 // Eight values at once.  A group without negative ones takes a shorter form
 // (the integer pipe, 16 lanes per clock and scheduler, is the bound: 11
 // instructions there and four wide products on the FMA pipe per value; shifts,
-// selects and a carry chain per value were 5% slower); both factors are 0 for a value outside the window (a zero, mostly), and what the
-// window missed is seen to afterwards.
+// selects and a carry chain per value were 5% slower); both factors are 0 for a
+// value outside the window (a zero, mostly), and what the window missed is seen
+// to afterwards.
 __device__ __forceinline__ void window_add8(Window& w, Parts& p, const double (&v)[8],
                                             long long* limbs, int* bad) {
   uint32_t any = 0u;

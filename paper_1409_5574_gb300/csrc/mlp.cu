@@ -34,7 +34,7 @@ namespace {
 constexpr int kTB = 128;  // samples per block (one tile: one sample per thread)
 
 // Canonical K-major strides (bytes per 8-row group) of the training tiles:
-// K = 64 (delta2 [s][j], W2^T [i][j]) and K = 128 (delta2^T [j][s], h1^T [i][s]).
+// K = 64 (delta2 [s][j], W2^T [i][j]) and K = 128 (h1^T [i][s]).
 constexpr uint32_t kTrSbo64 = (kHid / 8) * 128;
 constexpr uint32_t kTrSbo128 = (kTB / 8) * 128;
 

@@ -643,7 +643,7 @@ void free_sort(SortBuffers& b) {
 // against 318 us, of 16 steps 508 against 449; 2^21, 16 steps in launches of
 // one, two and four 1324 against 2040, 1158 against 1452 and 1059 against 1146
 // (in random order 4582 against 2086, 4570 and 4579 against 1503 and 1215; 8
-// steps in launches of one, 2^22 in cell order 1328 against 1777).  So launches of
+// steps in launches of one, 2^22 in cell order 1311 against 1777).  So launches of
 // fewer than kBinOrdered steps, and calls of less than 4 kBinMinWork, leave
 // particles to the plain kernel that follow an order of cells on the device's
 // count: more than half within near cells of the one before them, 8 for launches

@@ -1,11 +1,11 @@
 // Counting sort of particles by the 32 x 32-cell tile of the 2D Yee grid that
-// holds them and by cell inside each tile, and the work list of the tile-staged gather kernel: one
-// item per chunk of at most kChunk particles of one tile.  In cell order the
-// lanes of a warp read the same or neighbouring stencil values of the staged
-// tile (broadcasts instead of shared-memory bank conflicts).  Particles keep
-// their ids (pid array), so the Philox streams and ledger entries follow
-// them.  The order inside a cell depends on atomic timing; results per
-// particle do not.
+// holds them and by cell inside each tile, and the work list of the tile-staged
+// gather kernel: one item per chunk of at most kChunk particles of one tile.  In
+// cell order the lanes of a warp read the same or neighbouring stencil values
+// of the staged tile (broadcasts instead of shared-memory bank conflicts).
+// Particles keep their ids (pid array), so the Philox streams and ledger
+// entries follow them.  The order inside a cell depends on atomic timing;
+// results per particle do not.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(kCellThreads)
 // FP32, binning: a copy of the state in that order, on which the tile-staged
 // kernel runs.  It goes back to where it came from (particles that stay in
 // the caller's order) or, for the sorted path, in its own order, both streams
-// of whole lines.  The caller's arrays are only ever streamed; the scattered side is the copy, whose particles are
-// one 32-byte sector each.  (Gathering the seven arrays through an index in
+// of whole lines.  The caller's arrays are only ever streamed; the scattered
+// side is the copy, whose particles are one 32-byte sector each.  (Gathering the seven arrays through an index in
 // the push itself cost 0.25 ns per particle and launch on 8M particles in
 // random order; now 2^21 particles in random order take 13 us to count, 6 to
 // scan, 27 + 28 to place by tile and cell, 39 to copy and 26 to write back,
