@@ -1048,18 +1048,14 @@ __device__ __forceinline__ void advance_particle(const StepParams<R>& P, const u
   // Three or more outgrow the registers; the Yee step is too long for two (2^22
   // sorted electrons 8331 against 8370 us), and so is the batched kernel's, whose
   // parameters take registers (64 ensembles 3690 against 3712 us; it and the
-  // control kernels without the spread share the staging by field).  Kernels
-  // compiled at run time keep one: a second step gains 190 us per 100 steps of
-  // 2^24 electrons (15510 against 15710), and costs the context's first call 75
-  // ms of compilation, which a run of 4000 steps does not win back.
-#ifdef PRAD_SPEC
-  constexpr int kUnroll = 1;
-#else
+  // control kernels without the spread share the staging by field).  For kernels
+  // compiled at run time a second step gains 190 us per 100 steps of 2^24
+  // electrons (15510 against 15710) and costs the context's first call 60 to 75 ms
+  // of compilation.
   constexpr int kUnroll = sizeof(R) == 4 && FIELD != PRAD_FIELD_YEE2D &&
                                   !std::is_same<ST, PhotonStageSoA>::value
                               ? 2
                               : 1;
-#endif
 #pragma unroll kUnroll
   for (int s = 0; s < nsub; ++s) {
     const uint32_t step = static_cast<uint32_t>(P.t0 + s);
