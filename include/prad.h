@@ -122,7 +122,7 @@ typedef struct prad_config {
                                time by NVRTC with this context's constants
                                (time step, wave or grid geometry, Philox key
                                ...) as literals: the same results, fewer
-                               loads.  Each variant is compiled (~0.3-0.7 s)
+                               loads.  Each variant is compiled (~0.2-0.3 s)
                                at its first launch and kept until
                                prad_destroy; every distinct set of constants
                                (prad_set_fields with another wave or grid)
