@@ -32,13 +32,19 @@ def _problem(nx, ny, n, ex, ey, order=None, jitter=0.0):
     return wl
 
 
-def _run(wl, calls, per_launch, **kw):
-    ctx = prad.Context(wl.problem_kwargs(), photon_capacity=1 << 24, max_particles=wl.n,
+def _run(wl, calls, per_launch, ids=False, ledger=False, **kw):
+    problem = dict(wl.problem_kwargs())
+    if ledger:
+        problem["rr_mode"] = prad.PRAD_RR_LEDGER
+    ctx = prad.Context(problem, photon_capacity=1 << 24, max_particles=wl.n + 5,
                        steps_per_launch=per_launch, **kw)
     st = ctx.to_device(wl.state)
+    if ids:  # in another order than the particles
+        order = np.random.default_rng(1).permutation(wl.n).astype(np.int32)
+        st["pid"] = torch.as_tensor(order + 11).cuda()
     t = 0
     for steps in calls:
-        ctx.push_emit(st, steps, t0=t)
+        ctx.push_emit(st, steps, t0=t, pid0=11 if ids else 0, ledger_offset=5 if ids else 0)
         t += steps
     ph = ctx.photons(on_device=False)
     rec = np.stack([ph[k].numpy().view(np.uint32) for k in
@@ -62,6 +68,14 @@ CASES = {
     "cells, specialised": (2050, 2049, 2_097_152, 500, 500, "cells", 0.3, 9, 4, dict(specialize=True)),
     "random, specialised": (500, 490, 2_097_152, 500, 490, None, 0.0, 9, 4, dict(specialize=True)),
     "cells, short": (96, 130, 524_301, 96, 130, "cells", 0.0, 9, 9, {}),
+    "dense, control": (300, 280, 2_097_152, 300, 280, None, 0.0, 9, 9,
+                       dict(n_try=2, select_prob=0.5)),
+    "dense, ledger, ids": (300, 280, 2_097_157, 300, 280, None, 0.0, 9, 8,
+                           dict(ledger=True, ids=True)),
+    "one step, ledger, ids": (300, 280, 2_097_157, 300, 280, None, 0.0, 9, 1,
+                              dict(ledger=True, ids=True)),
+    "cells, one step, control": (300, 280, 2_097_157, 300, 280, "cells", 0.0, 9, 1,
+                                 dict(n_try=2, select_prob=0.5)),
     "more tiles than work": (8200, 8190, 524_301, 60, 70, None, 0.0, 8, 8, {}),
 }
 
@@ -72,7 +86,7 @@ def test_route_equals_one_step_calls(name):
         pytest.skip("no CUDA device")
     nx, ny, n, ex, ey, order, jitter, steps, per_launch, kw = CASES[name]
     wl = _problem(nx, ny, n, ex, ey, order, jitter)
-    a = _run(wl, [1] * steps, 1)
+    a = _run(wl, [1] * steps, 1, **{k: v for k, v in kw.items() if k != "specialize"})
     b = _run(wl, [steps], per_launch, **kw)
     for k in a[0]:
         np.testing.assert_array_equal(a[0][k], b[0][k], err_msg=k)
